@@ -65,81 +65,184 @@ struct NoallocCtl {
     double mx;              // max |r_i|
 };
 
-// One sweep, one thread per row, on a CSR matrix that stores its diagonal:
-//   s_i = sum_{j != i} a_ij x_j (stored order),  x'_i = (b_i - s_i) / a_ii,
-//   r_i = (b_i - s_i) - a_ii x_i,
-// with the residual sums (and ||b||^2, from the b_i each thread reads anyway)
-// reduced by the last block to finish, in block order.
-__global__ void __launch_bounds__(kBlock) k_noalloc_sweep(int n, const int* __restrict__ rowptr,
-                                                          const int* __restrict__ col,
-                                                          const double* __restrict__ val,
-                                                          const double* __restrict__ b,
-                                                          const double* __restrict__ x,
-                                                          double* __restrict__ y, unsigned char* scratch)
+// The larger of two magnitudes; a NaN wins.
+__device__ __forceinline__ double max_nan(double v, double m)
 {
-    double* part = reinterpret_cast<double*>(scratch + kOffPartial);
-    NoallocCtl* ctl = reinterpret_cast<NoallocCtl*>(scratch + kOffCtl);
+    return (v > m || v != v) ? v : m;
+}
+
+// Sums over a block, valid in thread 0: warp shuffle trees, then the warps'
+// sums in order.
+__device__ __forceinline__ void block_sums(double& ss, double& mx, double& bb)
+{
     __shared__ double s_ss[kBlock / 32], s_mx[kBlock / 32], s_bb[kBlock / 32];
-    __shared__ int s_last;
-    const int i = blockIdx.x * kBlock + threadIdx.x;
-    double ssq = 0.0, amx = 0.0, bsq = 0.0;
-    if (i < n) {
-        double s = 0.0, d = 0.0;
-        for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-            const int j = col[e];
-            if (j == i) d = val[e];
-            else s = __fma_rn(val[e], x[j], s);
-        }
-        const double bi = b[i];
-        bsq = bi * bi;
-        const double t = bi - s;
-        y[i] = t / d;
-        const double r = __fma_rn(-d, x[i], t);
-        ssq = r * r;
-        amx = fabs(r);
-        // a zero or missing diagonal, or an overflow, is reported as NaN
-        if (d == 0.0 || !(amx <= 1.7976931348623157e308)) amx = __longlong_as_double(0x7ff8000000000000ll);
-    }
     for (int o = 16; o > 0; o >>= 1) {
-        ssq += __shfl_down_sync(0xffffffffu, ssq, o);
-        bsq += __shfl_down_sync(0xffffffffu, bsq, o);
-        const double m = __shfl_down_sync(0xffffffffu, amx, o);
-        amx = (m > amx || m != m) ? m : amx;
+        ss += __shfl_down_sync(0xffffffffu, ss, o);
+        bb += __shfl_down_sync(0xffffffffu, bb, o);
+        mx = max_nan(__shfl_down_sync(0xffffffffu, mx, o), mx);
     }
     if ((threadIdx.x & 31) == 0) {
-        s_ss[threadIdx.x >> 5] = ssq;
-        s_mx[threadIdx.x >> 5] = amx;
-        s_bb[threadIdx.x >> 5] = bsq;
+        s_ss[threadIdx.x >> 5] = ss;
+        s_mx[threadIdx.x >> 5] = mx;
+        s_bb[threadIdx.x >> 5] = bb;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, m = 0.0, c = 0.0;
-        for (int w = 0; w < kBlock / 32; ++w) {
-            a += s_ss[w];
-            c += s_bb[w];
-            m = (s_mx[w] > m || s_mx[w] != s_mx[w]) ? s_mx[w] : m;
+    if (threadIdx.x == 0)
+        for (int w = 1; w < kBlock / 32; ++w) {
+            ss += s_ss[w];
+            bb += s_bb[w];
+            mx = max_nan(s_mx[w], mx);
         }
-        part[blockIdx.x] = a;
-        part[kMaxBlocks + blockIdx.x] = m;
-        part[2 * kMaxBlocks + blockIdx.x] = c;
-        __threadfence();
-        s_last = (atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (s_last && threadIdx.x == 0) {
-        __threadfence();
-        double a = 0.0, m = 0.0, c = 0.0;
-        for (unsigned q = 0; q < gridDim.x; ++q) {
-            a += part[q];
-            c += part[2 * kMaxBlocks + q];
-            const double v = part[kMaxBlocks + q];
-            m = (v > m || v != v) ? v : m;
+}
+
+// Entries staged at a time: a block's 256 rows of up to 7 entries in one
+// round (21.5 KB, eight blocks an SM); longer rows take several rounds.
+constexpr int kCap = 7 * kBlock;
+constexpr int kGather = 8;   // x loads of a row issued together
+
+__device__ __forceinline__ unsigned shared_addr(const void* p)
+{
+    return (unsigned)__cvta_generic_to_shared(p);
+}
+
+// One sweep on a CSR matrix that stores its diagonal, one thread per row:
+//   s_i = sum_{j != i} a_ij x_j (stored order),  x'_i = (b_i - s_i) / a_ii,
+// and in the last sweep of a call (LAST) also
+//   r_i = (b_i - s_i) - a_ii x_i
+// with the residual sums and ||b||^2 reduced by the last block to finish, in
+// a fixed order: the call returns those of its last sweep only, so the
+// sweeps before it compute none (each takes three more FP64 operations per
+// row and a reduction on a chip whose FP64 pipe is the co-bottleneck).
+//
+// A block copies its rows' entries into shared memory with coalesced
+// asynchronous copies of one entry each (the caller's arrays have no more
+// than their types' alignment), then each thread walks its row there: a
+// thread reading its 56-byte row straight from memory makes every warp load
+// touch 14 lines.  The copies, which read nothing that a sweep writes, start
+// before griddepcontrol.wait: the launches of a call depend on one another
+// programmatically, so a sweep's matrix is already arriving while the sweep
+// before it drains.
+template <bool LAST>
+__global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* __restrict__ rowptr,
+                                                             const int* __restrict__ col,
+                                                             const double* __restrict__ val,
+                                                             const double* __restrict__ b, const double* x, double* y,
+                                                             unsigned char* scratch)
+{
+    __shared__ double s_val[kCap];
+    __shared__ int s_col[kCap];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int r0 = blockIdx.x * kBlock, i = r0 + threadIdx.x;
+    const int p0 = rowptr[r0], p1 = rowptr[r0 + kBlock < n ? r0 + kBlock : n];
+    const int kb = i < n ? rowptr[i] : 0, ke = i < n ? rowptr[i + 1] : 0;
+    const double bi = i < n ? b[i] : 0.0;
+    double s = 0.0, d = 0.0, xi = 0.0;
+    bool waited = false;
+    for (int c0 = p0; c0 < p1 || !waited; c0 += kCap) {
+        const int c1 = p1 - c0 < kCap ? p1 : c0 + kCap;
+        if (waited) __syncthreads();        // the round before has been read
+#pragma unroll
+        for (int q = 0; q < kCap; q += kBlock) {
+            const int at = q + threadIdx.x, e = c0 + at;
+            if (e < c1) {
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(shared_addr(s_val + at)), "l"(val + e)
+                             : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(shared_addr(s_col + at)), "l"(col + e)
+                             : "memory");
+            }
         }
-        ctl->ss = a;
-        ctl->mx = m;
-        ctl->bb = c;
-        ctl->ticket = 0;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+        waited = true;
+        __syncthreads();
+        // this thread's part of the round; the loop ends at the warp's longest
+        const int lo = kb > c0 ? kb : c0, hi = ke < c1 ? ke : c1;
+        const int len = hi > lo ? hi - lo : 0;
+        const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
+        for (int o = 0; o < most; o += kGather) {
+            double xv[kGather];
+            int j[kGather];
+#pragma unroll
+            for (int u = 0; u < kGather; ++u) {
+                j[u] = i;
+                if (o + u < len) {
+                    j[u] = s_col[lo - c0 + o + u];
+                    xv[u] = x[j[u]];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kGather; ++u) {
+                if (o + u >= most) break;
+                if (o + u < len && j[u] == i) {
+                    d = s_val[lo - c0 + o + u];
+                    xi = xv[u];
+                }
+                // a warp whose rows all have their diagonal here skips the FMA
+                if (__any_sync(0xffffffffu, j[u] != i) && j[u] != i) s = __fma_rn(s_val[lo - c0 + o + u], xv[u], s);
+            }
+        }
     }
+    const double t = bi - s;
+    if (i < n) y[i] = t / d;
+    if constexpr (LAST) {
+        double ss = 0.0, mx = 0.0, bb = 0.0;
+        if (i < n) {
+            bb = bi * bi;
+            const double r = __fma_rn(-d, xi, t);
+            ss = r * r;
+            mx = fabs(r);
+            // a zero or missing diagonal, or an overflow, is reported as NaN
+            if (d == 0.0 || !(mx <= 1.7976931348623157e308)) mx = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        double* part = reinterpret_cast<double*>(scratch + kOffPartial);
+        NoallocCtl* ctl = reinterpret_cast<NoallocCtl*>(scratch + kOffCtl);
+        __shared__ int s_last;
+        block_sums(ss, mx, bb);
+        if (threadIdx.x == 0) {
+            part[blockIdx.x] = ss;
+            part[kMaxBlocks + blockIdx.x] = mx;
+            part[2 * kMaxBlocks + blockIdx.x] = bb;
+            __threadfence();
+            s_last = (atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1);
+        }
+        __syncthreads();
+        if (s_last) {
+            // the whole last block adds the blocks' sums, thread-strided then the
+            // block's tree (one thread alone took 3 ms for 13,000 blocks)
+            __threadfence();
+            ss = mx = bb = 0.0;
+            for (unsigned q = threadIdx.x; q < gridDim.x; q += kBlock) {
+                ss += __ldcg(part + q);
+                mx = max_nan(__ldcg(part + kMaxBlocks + q), mx);
+                bb += __ldcg(part + 2 * kMaxBlocks + q);
+            }
+            block_sums(ss, mx, bb);
+            if (threadIdx.x == 0) {
+                ctl->ss = ss;
+                ctl->mx = mx;
+                ctl->bb = bb;
+                ctl->ticket = 0;
+            }
+        }
+    }
+}
+
+cudaError_t launch_sweep(bool first, bool last, int n, const int* rowptr, const int* col, const double* val,
+                         const double* b, const double* x, double* y, unsigned char* scratch, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n + kBlock - 1) / kBlock));
+    cfg.blockDim = dim3(kBlock);
+    cfg.stream = s;
+    // a call's first sweep waits for everything before it on the stream, the
+    // others' prologues overlap the sweep before them
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = first ? 0 : 1;
+    return last ? cudaLaunchKernelEx(&cfg, k_noalloc_sweep<true>, n, rowptr, col, val, b, x, y, scratch)
+                : cudaLaunchKernelEx(&cfg, k_noalloc_sweep<false>, n, rowptr, col, val, b, x, y, scratch);
 }
 
 std::mutex g_mu;
@@ -221,7 +324,6 @@ try {
     }
     cudaStream_t s = (cudaStream_t)stream;
     const int nn = (int)n;
-    const int blocks = (int)((n + kBlock - 1) / kBlock);
     double* xs = reinterpret_cast<double*>(scratch);
     // the ticket must start at zero: a previous call may have been interrupted
     e = cudaMemsetAsync(scratch + kOffCtl, 0, sizeof(NoallocCtl), s);
@@ -231,8 +333,7 @@ try {
     const double* src = x_in;
     for (int i = 0; i < k && e == cudaSuccess; ++i) {
         double* dst = ((k - 1 - i) % 2 == 0) ? x_out : xs;
-        k_noalloc_sweep<<<blocks, kBlock, 0, s>>>(nn, rowptr, col, val, b, src, dst, scratch);
-        e = cudaGetLastError();
+        e = launch_sweep(i == 0, i == k - 1, nn, rowptr, col, val, b, src, dst, scratch, s);
         src = dst;
     }
     NoallocCtl h;
