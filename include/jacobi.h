@@ -142,15 +142,17 @@ typedef struct {
                                   Sec. 4.2.2) staged into shared memory */
     int32_t tile_rows;         /* threads of a tile (one row each when lanes_per_row = 1): 0 = auto
                                   (256), 224, 256 or 480 (variant 2); 256 (variant 3) */
-    int32_t ctas_per_sm;       /* variant 2 with 256-row tiles: 0 = auto (2), or 3 (3-stage pipeline) */
+    int32_t ctas_per_sm;       /* variant 2 with 256-row tiles: 2, 3 (3-stage pipeline), or 0 = auto (by the
+                                  row length, the precision and n where stages is 0 too, else 2) */
     int32_t lanes_per_row;     /* variant 2 with 256-thread tiles: lanes summing one row (1, 2, 4, 8);
                                   0 = auto: the smallest count whose tile of 256/L longest rows fits a
                                   pipeline stage.  Each row is summed by L interleaved FMA chains and
                                   a fixed pairwise tree, so iterates are bit-identical across
                                   splittings and tilings for a given L and agree to rounding
                                   across L. */
-    int32_t stages;            /* variant 2, 256 threads, 2 CTAs/SM: pipeline stages 0 = auto (4), or 3 / 2
-                                  larger stages (36 / 54 KB) that hold whole tiles of long rows */
+    int32_t stages;            /* variant 2, 256 threads, 2 CTAs/SM: pipeline stages, 4, or 3 / 2 larger
+                                  stages (36 / 54 KB) that hold whole tiles of long rows; 0 = auto (as
+                                  ctas_per_sm; 4 where that is given) */
     int32_t sync;              /* jac_sync (default JAC_SYNC_GRID; the autotuner tries grid and
                                   neighbour; JAC_SYNC_ASYNC only when asked for) */
     int32_t debug;             /* 1: canary bytes in the 16-element padding after every device vector of

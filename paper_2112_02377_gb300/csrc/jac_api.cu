@@ -880,6 +880,24 @@ try {
 
 inline int64_t nnz_off_of(const ScaledForm& tf) { return tf.rowptr.empty() ? 0 : tf.rowptr.back(); }
 
+// CTAs per SM and pipeline stages (0: the default 4) where the caller leaves
+// both open.  Measured on GB300, us per sweep without calibration:
+//   one lane per row (7-point), 2 against 3 CTAs/SM: a third CTA hides more of
+//     the gathers' latency and costs a longer grid barrier.  FP64: 64^3 10.7 /
+//     11.8, 128^3 37.3 / 37.3, 160^3 70.2 / 66.1; a mixed cycle's FP32 sweeps
+//     (bound by that latency) from about 100,000 rows on: 48^3 4.03 / 3.98, 96^3
+//     13.0 / 10.6, 128^3 25.9 / 21.3, 160^3 48.2 / 38.9;
+//   several lanes (27-point), 4 / 3 / 2 stages: a 26 KB stage holds 78 of the 128
+//     rows of a two-lane tile, a 54 KB one all.  FP64: 32^3 9.6 / 9.5 / 8.6, 64^3
+//     24.5 / 24.3 / 20.7, 128^3 152 / 139 / 127; mixed 48^3 7.1 / 6.6 / 5.8, 64^3
+//     13.6 / 11.7 / 11.5, 96^3 40.7 / 34.7 / 39.0 (FP32 entries take two thirds
+//     of the space, and 36 KB hold the tile).
+static void default_geometry(int lanes, bool mixed, int64_t rows, int* per_sm, int* stages)
+{
+    if (lanes == 1) *per_sm = rows >= (mixed ? 100000 : 3000000) ? 3 : 2;
+    else *stages = mixed && rows > 350000 ? 3 : 2;
+}
+
 // A context from a matrix already split and scaled: tf holds the kernel rows
 // (tf.n of them; n for jac_setup, more with a split interface block), tf.d and
 // the iterate the n rows.  sp: the split interface layout (jac_setup_local),
@@ -922,18 +940,12 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     CK(nullptr, cudaGetDeviceProperties(&prop, dev));
     Tiling tl;
     Windows win;
-    // Default geometry: the persistent kernel with 8 math warps (256 threads),
-    // 2 CTAs/SM and the plain row loop; the autotuner also tries 3 CTAs/SM
-    // and the 7/15-warp software-pipelined geometries.
+    // Default geometry: the persistent kernel with 8 math warps (256 threads);
+    // the autotuner also tries the 7/15-warp software-pipelined geometries.
     c->variant = o.variant == 0 ? 2 : o.variant;
     c->rows_per_tile = o.tile_rows ? o.tile_rows : 256;
     c->stages = 4;
     if (c->variant == 3 && c->rows_per_tile != 256) c->variant = 2;
-    const int target_per_sm = (c->variant == 2 && c->rows_per_tile == 256 && o.ctas_per_sm == 3) ? 3 : 2;
-    if (target_per_sm == 3) c->stages = 3;
-    // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
-    if (c->variant == 2 && c->rows_per_tile == 256 && target_per_sm == 2 && (o.stages == 2 || o.stages == 3))
-        c->stages = o.stages;
     // Lanes per row (256-thread geometry only): long rows fill a stage's
     // entry budget with few rows, which leaves math warps without a row, and
     // a long FMA chain per thread; L lanes per row split both.  Each lane's
@@ -950,6 +962,15 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     } else if (o.lanes_per_row > 1) {
         return fail(nullptr, JAC_EINVAL, "opts.lanes_per_row > 1 needs variant 2 with 256-thread tiles");
     }
+    int target_per_sm = (c->variant == 2 && c->rows_per_tile == 256 && o.ctas_per_sm == 3) ? 3 : 2;
+    int stages = o.stages;
+    if (c->variant == 2 && c->rows_per_tile == 256 && !o.ctas_per_sm && !o.stages && o.sync == JAC_SYNC_GRID &&
+        o.stop == JAC_STOP_GLOBAL)
+        default_geometry(c->lanes, o.precision == JAC_MIXED, rows, &target_per_sm, &stages);
+    if (target_per_sm == 3) c->stages = 3;
+    // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
+    if (c->variant == 2 && c->rows_per_tile == 256 && target_per_sm == 2 && (stages == 2 || stages == 3))
+        c->stages = stages;
     if (c->variant >= 2) {
         const int rows = c->rows_per_tile / c->lanes;     // rows of a tile
         int64_t cap_entries = (int64_t)std::max<int64_t>(1, tf.max_off) * rows;
