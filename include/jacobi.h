@@ -128,7 +128,8 @@ typedef struct {
 typedef struct {
     int32_t precision;         /* jac_precision (default JAC_FP64) */
     int32_t norm;              /* jac_norm (default JAC_NORM_REL2) */
-    int32_t sweeps_per_graph;  /* sweeps per CUDA-graph launch, 1..4096 (default 64) */
+    int32_t sweeps_per_graph;  /* sweeps per CUDA-graph launch, 1..4096 (default 64; at least 512 where the
+                                  matrix is kept in shared memory, see variant) */
     int32_t inner_sweeps;      /* JAC_MIXED: FP32 sweeps per FP64 refinement step, >= 1 (default 128) */
     int32_t grid[3];           /* node grid (gx, gy, gz); required for JAC_SUBSTRUCT */
     int32_t subdomains[3];     /* boxes per axis (px, py, pz); JAC_SUBSTRUCT only */
@@ -136,7 +137,10 @@ typedef struct {
                                   NULL = row r sits at node r */
     int32_t nrhs;              /* right-hand sides sharing A (1..8, default 1) */
     int32_t transpose;         /* 1 = solve with A^T instead of A (adjoint solves) */
-    int32_t variant;           /* 0 = auto (2); 1 = one launch per sweep (row kernel);
+    int32_t variant;           /* 0 = auto: 2, or, in FP64 with the grid barrier, the global stop, 1 or 2 lanes
+                                  per row and no other geometry option, where the matrix fits the
+                                  SMs' shared memory, a kernel that keeps it there (jac_stats:
+                                  variant 2, ctas_per_sm 1, stages 0); 1 = one launch per sweep (row kernel);
                                   2 = persistent grid-synchronised pipelined kernel, x gathered
                                   through L1/L2; 3 = as 2 with each tile's x halo (its dependency list,
                                   Sec. 4.2.2) staged into shared memory */

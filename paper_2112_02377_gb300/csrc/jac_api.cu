@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <stdexcept>
 #include <numeric>
@@ -51,8 +52,10 @@ struct jac_ctx {
     float* d_S32 = nullptr;
     double* d_b = nullptr;         // b in the new row order (FP64 sweep input)
     double* d_d = nullptr;
-    double* d_x[3] = {nullptr, nullptr, nullptr};
-    int nbuf = 2;                  // iterate buffers in rotation (3 with neighbour sync)
+    double* d_x[4] = {nullptr, nullptr, nullptr, nullptr};
+    int nbuf = 2;                  // iterate buffers in rotation (3 with neighbour sync, 4 in the resident kernel)
+    bool resident = false;         // FP64 sweeps run in the resident kernel
+    int* d_cta_row = nullptr;      // resident kernel: ctas+1 first rows
     bool ns = false;               // neighbour-synchronised FP64 sweeps
     int sync = JAC_SYNC_GRID;      // jac_sync of the FP64 kernel
     bool certify = false;          // asynchronous contexts: run the grid-synchronised kernel
@@ -236,6 +239,19 @@ void dfree(T*& p)
 
 cudaStream_t stream_of(const jac_ctx* c) { return c->stream; }
 
+// Lets kernel `fn` be launched with `bytes` of dynamic shared memory.  The limit
+// belongs to the kernel, which several contexts share: it is only ever raised.
+cudaError_t allow_smem(const void* fn, int bytes)
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lk(mu);
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, fn);
+    if (e == cudaSuccess && a.maxDynamicSharedSizeBytes < bytes)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
+}
+
 jac_status copy_to_stage(jac_ctx* c, const double* src, int memory, size_t count, double* stage)
 {
     if (memory == JAC_MEM_DEVICE) {
@@ -282,6 +298,7 @@ DevVec devvec(const jac_ctx* c)
     v.x[0] = c->d_x[0];
     v.x[1] = c->d_x[1];
     v.x[2] = c->d_x[2];
+    v.x[3] = c->d_x[3];
     v.nbuf = c->nbuf;
     v.e[0] = c->d_e[0];
     v.e[1] = c->d_e[1];
@@ -349,6 +366,11 @@ int mixed_cycles_per_step(const jac_ctx* c)
     return std::max(1, (c->K + m - 1) / m);
 }
 
+// FP64 sweeps of a graph step.  The resident kernel loads the matrix and ends
+// with a barrier of its own in every launch (about 10 us together), against 2 us
+// a sweep: its steps have at least 512 sweeps.
+int sweeps_per_step(const jac_ctx* c) { return c->resident ? std::max(c->K, 512) : c->K; }
+
 // Enqueue one "graph step": K sweeps (FP64) or one refinement cycle block (mixed).
 jac_status enqueue_step(jac_ctx* c, bool mixed)
 {
@@ -368,6 +390,12 @@ jac_status enqueue_step(jac_ctx* c, bool mixed)
                 CK(c, launch_batched(fn, c->grid, c->threads, c->smem, devmat(c), devvec(c), devtiles(c),
                                      devbatch(c), c->d_ctl, c->o.inner_sweeps, s));
             }
+        return JAC_OK;
+    }
+    if (c->resident) {
+        CK(c, launch_reset_bar(c->d_ctl, s));
+        CK(c, launch_resident(c->pfn64, c->grid, c->smem, devmat(c), devvec(c), c->d_cta_row, c->d_ctl,
+                              sweeps_per_step(c), s));
         return JAC_OK;
     }
     if (c->variant >= 2) {
@@ -546,7 +574,7 @@ void destroy(jac_ctx* c)
     if (c->ev0) cudaEventDestroy(c->ev0);
     if (c->ev1) cudaEventDestroy(c->ev1);
     dfree(c->d_rowptr); dfree(c->d_col); dfree(c->d_S64); dfree(c->d_S32); dfree(c->d_b); dfree(c->d_d);
-    dfree(c->d_x[0]); dfree(c->d_x[1]); dfree(c->d_x[2]);
+    dfree(c->d_x[0]); dfree(c->d_x[1]); dfree(c->d_x[2]); dfree(c->d_x[3]); dfree(c->d_cta_row);
     dfree(c->d_dep_ptr); dfree(c->d_dep); dfree(c->d_done); dfree(c->d_e[0]); dfree(c->d_e[1]); dfree(c->d_dlt);
     dfree(c->d_part); dfree(c->d_ctl); dfree(c->d_hist); dfree(c->d_perm); dfree(c->d_stage); dfree(c->d_stage2);
     dfree(c->d_bmap); dfree(c->d_slot_info);
@@ -898,6 +926,29 @@ static void default_geometry(int lanes, bool mixed, int64_t rows, int* per_sm, i
     else *stages = mixed && rows > 350000 ? 3 : 2;
 }
 
+// Row ranges of the resident kernel's CTAs and the dynamic shared memory of the
+// largest; 0 if a row is too long for it.  It is used wherever it fits: measured
+// on GB300, us per sweep, pipelined / resident: 7-point 8^3 6.8 / 2.7, 32^3 6.9 /
+// 2.9, 48^3 8.4 / 3.7, 64^3 10.7 / 6.0, 70^3 12.0 / 7.1 (74^3 does not fit);
+// 27-point 16^3 7.5 / 2.8, 32^3 8.6 / 4.5, 44^3 11.7 / 7.5 (48^3 does not fit).
+static int64_t resident_plan(const ScaledForm& tf, const Plan& plan, int ctas, int lanes,
+                             const std::vector<double>* row_cost, std::vector<int32_t>& cut)
+{
+    // cheap bound first: entries, b, the iterate and the counts of an even share
+    if ((12.0 * tf.rowptr[tf.n] + 18.0 * tf.n) / ctas > 227.0 * 1024) return 0;
+    Tiling t;
+    make_tiling(tf, plan, 1 << 30, 1 << 30, ctas, t, row_cost);
+    cut.resize(ctas + 1);
+    int64_t most = 0;
+    for (int g = 0; g <= ctas; ++g) cut[g] = t.row0[t.cta0[g]];
+    for (int g = 0; g < ctas; ++g) {
+        const int64_t b = resident_smem_bytes(tf.rowptr.data(), cut[g], cut[g + 1], lanes);
+        if (b < 0) return 0;
+        most = std::max(most, b);
+    }
+    return most;
+}
+
 // A context from a matrix already split and scaled: tf holds the kernel rows
 // (tf.n of them; n for jac_setup, more with a split interface block), tf.d and
 // the iterate the n rows.  sp: the split interface layout (jac_setup_local),
@@ -971,7 +1022,34 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
     if (c->variant == 2 && c->rows_per_tile == 256 && target_per_sm == 2 && (stages == 2 || stages == 3))
         c->stages = stages;
-    if (c->variant >= 2) {
+    // ---- the resident kernel, where the caller leaves the geometry open and the matrix fits
+    bool all_auto = o.variant == 0 && !o.tile_rows && !o.ctas_per_sm && !o.stages;
+    if (all_auto && !sp && o.precision == JAC_FP64 && o.sync == JAC_SYNC_GRID && o.stop == JAC_STOP_GLOBAL &&
+        resident_kernel(c->lanes)) {
+        const int G = prop.multiProcessorCount;
+        std::vector<int32_t> cut;
+        const int64_t need = resident_plan(tf, plan, G, c->lanes, row_cost, cut);
+        int coop = 0, fits = 0;
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        const void* fn = resident_kernel(c->lanes);
+        if (need > 0 && need <= (int64_t)prop.sharedMemPerBlockOptin && coop &&
+            allow_smem(fn, (int)need) == cudaSuccess &&
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, fn, resident_threads(), (size_t)need) == cudaSuccess &&
+            fits >= 1) {
+            c->resident = true;
+            c->pfn64 = c->pfn64grid = fn;
+            c->grid = c->sms = G;
+            c->threads = resident_threads();
+            c->smem = (int)need;
+            c->stages = 0;
+            c->ntiles = G;
+            c->nbuf = 4;
+            c->h_cta_row0 = cut;
+        } else {
+            cudaGetLastError();
+        }
+    }
+    if (c->variant >= 2 && !c->resident) {
         const int rows = c->rows_per_tile / c->lanes;     // rows of a tile
         int64_t cap_entries = (int64_t)std::max<int64_t>(1, tf.max_off) * rows;
         int64_t stage_budget;
@@ -1014,7 +1092,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
             if (!c->pfn64 || (!c->pfnmix && !sp)) return 0;
             if (c->pfnmix32 && c->variant == 2) {
                 int a4 = 0;
-                if (cudaFuncSetAttribute(c->pfnmix32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) !=
+                if (allow_smem(c->pfnmix32, smem_bytes) !=
                         cudaSuccess ||
                     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a4, c->pfnmix32, c->threads, smem_bytes) !=
                         cudaSuccess || a4 < 1) {
@@ -1023,8 +1101,8 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
                 }
             }
             const void* fmix = c->pfnmix ? c->pfnmix : c->pfn64;
-            if (cudaFuncSetAttribute(c->pfn64, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess ||
-                cudaFuncSetAttribute(fmix, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) {
+            if (allow_smem(c->pfn64, smem_bytes) != cudaSuccess ||
+                allow_smem(fmix, smem_bytes) != cudaSuccess) {
                 cudaGetLastError();
                 return 0;
             }
@@ -1035,7 +1113,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
                 return 0;
             }
             if (c->pfn64grid && c->pfn64grid != c->pfn64 &&
-                (cudaFuncSetAttribute(c->pfn64grid, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) !=
+                (allow_smem(c->pfn64grid, smem_bytes) !=
                      cudaSuccess ||
                  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a3, c->pfn64grid, c->threads, smem_bytes) !=
                      cudaSuccess)) {
@@ -1101,16 +1179,19 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         }
         row_cost = &split_cost;
     }
-    if (c->variant == 2 && !sp) {
+    if (c->resident) {
+    } else if (c->variant == 2 && !sp) {
         make_tiling(tf, plan, c->rows_per_tile / c->lanes, c->emax, c->grid, tl, row_cost);
     } else if (c->variant == 2) {
         make_split_tiling(*sp, c->rows_per_tile / c->lanes, c->emax, c->grid, tl, row_cost);
     }
     if (c->variant >= 2) {
-        c->ntiles = (int)tl.ntiles();
         // what the balance calibration needs: each CTA's rows and the cost model used
-        c->h_cta_row0.resize(c->grid + 1);
-        for (int g = 0; g <= c->grid; ++g) c->h_cta_row0[g] = tl.row0[tl.cta0[g]];
+        if (!c->resident) {
+            c->ntiles = (int)tl.ntiles();
+            c->h_cta_row0.resize(c->grid + 1);
+            for (int g = 0; g <= c->grid; ++g) c->h_cta_row0[g] = tl.row0[tl.cta0[g]];
+        }
         c->h_cta_row1.clear();
         if (!tl.cta1.empty()) {
             c->h_cta_row1.resize(c->grid + 1);
@@ -1168,6 +1249,13 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         c->nbuf = 3;
         CK(nullptr, dalloc(&c->d_x[2], n + 16));
     }
+    if (c->resident) {
+        CK(nullptr, dalloc(&c->d_x[2], n + 16));
+        CK(nullptr, dalloc(&c->d_x[3], n + 16));
+        CK(nullptr, dalloc(&c->d_cta_row, (size_t)c->grid + 1));
+        CK(nullptr, cudaMemcpy(c->d_cta_row, c->h_cta_row0.data(), (c->grid + 1) * sizeof(int32_t),
+                               cudaMemcpyHostToDevice));
+    }
     if (o.precision == JAC_MIXED) {
         CK(nullptr, dalloc(&c->d_S32, nnz_off + 16));
         CK(nullptr, dalloc(&c->d_e[0], n + 16));
@@ -1219,7 +1307,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         CK(nullptr, cudaMemcpy(c->d_dep_ptr, dep_ptr.data(), dep_ptr.size() * 4, cudaMemcpyHostToDevice));
         if (!dep.empty()) CK(nullptr, cudaMemcpy(c->d_dep, dep.data(), dep.size() * 4, cudaMemcpyHostToDevice));
     }
-    if (c->variant >= 2) {
+    if (c->variant >= 2 && !c->resident) {
         CK(nullptr, dalloc(&c->d_row0, tl.row0.size()));
         CK(nullptr, dalloc(&c->d_nnz0, tl.nnz0.size()));
         CK(nullptr, dalloc(&c->d_cta0, tl.cta0.size()));
@@ -1267,6 +1355,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         add_canary(C, "x[0]", c->d_x[0], nn);
         add_canary(C, "x[1]", c->d_x[1], nn);
         add_canary(C, "x[2]", c->d_x[2], nn);
+        add_canary(C, "x[3]", c->d_x[3], nn);
         add_canary(C, "e[0]", c->d_e[0], nn);
         add_canary(C, "e[1]", c->d_e[1], nn);
         add_canary(C, "r (FP32)", c->d_dlt, nn);
@@ -1509,6 +1598,10 @@ try {
     // (short rows, FP64-pipe and gather bound); long rows (2+ lanes) with
     // 2 CTAs/SM and 2 large stages that hold whole tiles of 256/L rows.
     std::vector<Geometry> cand;
+    // (FP64 systems that fit the chip's shared memory: what an open geometry gives, the resident kernel)
+    if (o.precision == JAC_FP64 && !async && !local_stop && resident_kernel(la) && !o.stages &&
+        prep.tf.rowptr[prep.tf.n] <= 3000000)
+        cand.push_back({0, 0, 0, 0});
     if (la >= 2 && !async) cand.push_back({2, 256, 2, 0, JAC_SYNC_GRID, 2});
     else cand.push_back({2, 256, 3, 0});
     auto add = [&](const Geometry& g) {
@@ -1780,9 +1873,9 @@ try {
     c->threads = batched_threads(rows);
     int per_sm = 0;
     {
-        CK(nullptr, cudaFuncSetAttribute(c->pfn64, cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem));
-        CK(nullptr, cudaFuncSetAttribute(c->pfnmix, cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem));
-        CK(nullptr, cudaFuncSetAttribute(c->pfnmix32, cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem));
+        CK(nullptr, allow_smem(c->pfn64, c->smem));
+        CK(nullptr, allow_smem(c->pfnmix, c->smem));
+        CK(nullptr, allow_smem(c->pfnmix32, c->smem));
         int a1 = 0, a2 = 0, a3 = 0;
         CK(nullptr, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a1, c->pfn64, c->threads, c->smem));
         CK(nullptr, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a2, c->pfnmix, c->threads, c->smem));
@@ -1955,7 +2048,7 @@ try {
     }
     jac_status st = arm(c, 0, 0, 0, k, -1.0);
     if (st != JAC_OK) return st;
-    const int launches = (k + c->K - 1) / c->K;
+    const int launches = (int)(((int64_t)k + sweeps_per_step(c) - 1) / sweeps_per_step(c));
     CK(c, cudaEventRecord(c->ev0, s));
     for (int i = 0; i < launches; ++i) {
         st = run_graph(c, false);
@@ -2045,7 +2138,7 @@ static jac_status solve_impl(jac_ctx* c, double tol, int64_t maxit, int64_t* swe
     const long long per_step = (c->variant == 1 && mixed) ? c->o.inner_sweeps
                                : (mixed && (c->batched || c->pfnmix32))
                                    ? (long long)mixed_cycles_per_step(c) * std::max(2, c->o.inner_sweeps)
-                                                       : c->K;
+                                                       : sweeps_per_step(c);
     const long long step_cap = (maxit + (long long)c->o.inner_sweeps + 1) / per_step + 4;
     long long steps = 1;
     for (;;) {

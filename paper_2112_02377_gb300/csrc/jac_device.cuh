@@ -61,7 +61,7 @@ struct JacCtl {
     double loc_val;
 };
 
-struct Partial {
+struct alignas(16) Partial {
     double ss;                // sum of r_i^2
     unsigned long long mx;    // max over rows of abs_key(r_i)
 };
@@ -94,8 +94,8 @@ struct DevMat {
 };
 
 struct DevVec {
-    double* x[3];             // FP64 iterate y = D x: nbuf buffers used in rotation
-    int nbuf;                 // 2 (ping-pong) or 3 (neighbour-synchronised sweeps)
+    double* x[4];             // FP64 iterate y = D x: nbuf buffers used in rotation
+    int nbuf;                 // 2 (ping-pong), 3 (neighbour-synchronised sweeps) or 4 (resident kernel)
     float* e[2];              // FP32 inner iterate f = D e, ping-pong (mixed)
     float* dlt;               // FP32 residual r of the last P64R pass (mixed)
     Partial* part;            // [2][nslots] per-sweep partial norms
@@ -285,7 +285,7 @@ __device__ __forceinline__ int phase_of(bool mixed, int pos, int inner)
     return pos == inner - 1 ? PH_P32L : PH_P32;
 }
 
-// Fixed-order reduction of `cnt` partials by one warp (lane 0 gets the result).
+// Fixed-order reduction of `cnt` partials by one warp (every lane gets the result).
 __device__ __forceinline__ void reduce_partials_warp(const Partial* p, int cnt, double& ss,
                                                      unsigned long long& mx)
 {

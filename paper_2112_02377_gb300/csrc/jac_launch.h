@@ -16,6 +16,14 @@ cudaError_t launch_row_sweep(int phase, const DevMat& m, const DevVec& v, JacCtl
 const void* persistent_kernel(int threads, int stages, bool mixed, int lanes, int sync, int part = 0);
 int persistent_smem_bytes(int rows, int emax, int stages);
 int persistent_threads(int rows);
+// Resident kernel (one CTA per SM, matrix in shared memory): lanes per row 1 or
+// 2, else nullptr; cta_row: grid+1 first rows.  resident_smem_bytes: what rows
+// [r0, r1) need (negative: a row too long).
+const void* resident_kernel(int lanes);
+int resident_threads();
+long long resident_smem_bytes(const int* rowptr, int r0, int r1, int lanes);
+cudaError_t launch_resident(const void* fn, int grid, int smem, const DevMat& m, const DevVec& v, const int* cta_row,
+                            JacCtl* ctl, int max_sweeps, cudaStream_t s);
 const void* halo_kernel(int stages, bool mixed);
 int halo_smem_bytes(int rows, int emax, int xcap, int ntcap, int blkcap, int stages);
 cudaError_t launch_persistent(const void* fn, int grid, int threads, int smem, const DevMat& m, const DevVec& v,

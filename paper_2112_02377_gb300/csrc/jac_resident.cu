@@ -1,0 +1,399 @@
+// FP64 sweeps of systems whose matrix fits in the chip's shared memory.
+//
+// One CTA per SM keeps its rows of S, their columns, b and its part of the
+// iterate in shared memory for the whole launch; a sweep then moves only the
+// iterate, through L2.  What is left of such a sweep is latency, and this
+// kernel is arranged around the chain that every sweep has to go through:
+// gather x, sum the row, store, pass the grid barrier (fence, arrival, poll:
+// 1.3 us with one CTA per SM).  GB300's FP64 pipe takes 64 cycles per warp
+// instruction and sub-partition, so the residual norm -- shuffle trees of
+// FP64 adds, a square root, a division -- costs several times the row sums of
+// a small system.  It is taken off the chain altogether:
+//   sweep s      the math warps leave each thread's sum of r^2 and max |r| in
+//                shared memory;
+//   sweep s + 1  one spare warp adds them and publishes the CTA's partial sums;
+//   sweep s + 2  another spare warp adds all CTAs' partials (the barrier of
+//                sweep s + 1 made them visible) and takes the decision of sweep s.
+// The iterate rotates through four buffers, so the x^k that a stop returns is
+// still there two sweeps later; counts, results and histories are those of the
+// other kernels.
+//
+// Measured on GB300, 16^3 7-point: 2.75 us a sweep, of them 1.2 us in the grid
+// barrier (a bare one takes 1.4 us; splitting its counter over several lines or
+// polling differently changes less than 3 %); the pipelined kernel takes 7.0.
+// 64^3: 6.0 us against 10.7, of which 3.4 are the FP64 pipe's.  More sizes at the
+// rule in jac_api.cu (resident_plan).
+#include <cuda_runtime.h>
+
+#include "jac_device.cuh"
+#include "jac_launch.h"
+
+namespace jac {
+
+namespace {
+
+constexpr int MW = 16;                          // math warps
+constexpr int RT = (MW + 2) * 32;               // threads: math warps, then the two spare warps
+constexpr int CH = 8;                           // entries whose gathers are issued together
+
+struct ResidentDecision {
+    long long k, k_limit, hist_at, hist_cap;    // iterate of the launch's first sweep; limits
+    double tol, bnorm, pass;
+    double* hist;                               // CTA 0 only
+    int kind, test, done;
+    double relres, res2, resinf;
+    long long k_eval;
+};
+
+template <int ID>
+__device__ __forceinline__ void cta_sync()
+{
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(RT) : "memory");
+}
+
+__device__ void init_decision(ResidentDecision& d, const volatile JacCtl* c)
+{
+    d.k = c->k;
+    d.k_limit = c->k_limit;
+    d.hist_at = c->evals;
+    d.hist_cap = c->hist_cap;
+    d.tol = c->tol;
+    d.bnorm = c->bnorm;
+    d.hist = blockIdx.x == 0 ? c->hist : nullptr;
+    d.kind = c->norm_kind;
+    d.test = c->test;
+    d.done = DONE_RUNNING;
+    d.relres = c->relres;
+    d.res2 = c->res2;
+    d.resinf = c->resinf;
+    d.k_eval = c->k_eval;
+    // A sum of squares above this fails the 2-norm test whatever decide()
+    // rounds (the margin covers its roundings and ours), so most sweeps are
+    // decided without its square root and division.  Where the product is too
+    // small to carry the margin, decide() is always asked.
+    const double v = d.bnorm > 0.0 ? d.tol * d.bnorm : d.tol;
+    d.pass = v * v * (1.0 + 1e-12);
+    if (!(d.pass > 1e-280)) d.pass = 1.7976931348623157e308;
+}
+
+// The decision of sweep j of the launch, by one warp, from every CTA's partial sums.
+__device__ void take_decision(ResidentDecision& s, const Partial* part, JacCtl* ctl, int j, bool last)
+{
+    double tss;
+    unsigned long long tmx;
+    reduce_partials_warp(part, gridDim.x, tss, tmx);
+    if ((threadIdx.x & 31) == 0) {
+        const long long k = s.k + j;
+        int done = DONE_RUNNING;
+        const bool bad = !(tss <= 1.7976931348623157e308) || tmx >= KEY_INF;
+        const bool near = s.kind == 2 ? !(tss > s.pass) : abs_from_key(tmx) <= s.tol;
+        if (last || s.hist || bad || (s.test && (k >= s.k_limit || near))) {
+            const Decision d = decide(s.test, s.tol, s.k_limit, s.kind, s.bnorm, tss, tmx, k);
+            s.relres = d.relres;
+            s.res2 = d.res2;
+            s.resinf = d.resinf;
+            s.k_eval = k;
+            done = d.done;
+            if (d.numeric_bad && blockIdx.x == 0) atomicOr(&ctl->status, ST_NUMERIC);
+            if (s.hist && s.hist_at + j < s.hist_cap) s.hist[s.hist_at + j] = d.relres;
+        }
+        s.done = done;
+    }
+}
+
+// A CTA's partial sums of one sweep, by one warp: its math threads' sums
+// (active: those that own rows), lane-strided, then a fixed tree.
+__device__ void publish(const double* ss, const unsigned long long* mx, int active, Partial* slot)
+{
+    const int lane = threadIdx.x & 31;
+    double a = 0.0;
+    unsigned long long b = 0;
+    for (int i = lane; i < active; i += 32) {
+        a += ss[i];
+        b = umax64(b, mx[i]);
+    }
+    a = warp_sum(a);
+    b = warp_max(b);
+    if (lane == 0) {
+        __stcg(&slot->ss, a);
+        __stcg(&slot->mx, b);
+    }
+}
+
+}  // namespace
+
+// Dynamic shared memory of a CTA: `words` 12-byte entry slots (32 per entry
+// column of a slice), then b and the iterate of its rows, then each slice's
+// offset and the lanes' entry counts.  Slices are 32 / L rows.
+__host__ __device__ static inline long long resident_bytes(long long words, int rows, int slices)
+{
+    return words * 12 + 16ll * rows + 4ll * (slices + 1) + 64ll * slices + 32;
+}
+
+long long resident_smem_bytes(const int* rowptr, int r0, int r1, int lanes)
+{
+    const int rps = 32 / lanes;
+    const int slices = (r1 - r0 + rps - 1) / rps;
+    long long words = 0;
+    for (int s = 0; s < slices; ++s) {
+        int w = 0;
+        for (int r = r0 + s * rps; r < r1 && r < r0 + (s + 1) * rps; ++r) {
+            const int len = (rowptr[r + 1] - rowptr[r] + lanes - 1) / lanes;
+            w = len > w ? len : w;
+        }
+        if (w > 65535) return -1;
+        words += 32ll * w;
+    }
+    return resident_bytes(words, r1 - r0, slices);
+}
+
+// L lanes sum a row (1 or 2), as in the pipelined kernel: interleaved chains in
+// stored order, then the pairwise add, so the iterates are the same bits.
+//
+// Entries are stored slice by slice, entry-major (entry e of lane l at
+// 32 e + l): a warp's reads of S and col are consecutive.
+template <int L>
+__global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const int* __restrict__ cta_row, JacCtl* ctl,
+                                                    int max_sweeps)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ double s_ss[2][MW * 32];
+    __shared__ unsigned long long s_mx[2][MW * 32];
+    __shared__ ResidentDecision s_dec;
+    __shared__ int s_start, s_skip, s_xb, s_words;
+    __shared__ volatile int s_fail;
+    __shared__ long long s_budget;
+    __shared__ double* s_x[4];            // (indexed in shared memory: a local copy would be re-read from L2)
+    constexpr int RPS = 32 / L;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r0 = cta_row[blockIdx.x], rows = cta_row[blockIdx.x + 1] - r0;
+    const int ns = (rows + RPS - 1) / RPS;
+    if (tid == 0) {
+        const volatile JacCtl* c = ctl;
+        init_decision(s_dec, c);
+        s_xb = c->xbuf;
+        s_budget = c->timeout;
+        s_skip = c->fault_skip_cta;
+        s_start = c->done == DONE_RUNNING && c->status == 0;
+        s_fail = 0;
+        for (int q = 0; q < 4; ++q) s_x[q] = v.x[q];
+    }
+    // ---- slice offsets: widths first (kept in the offsets' place), then their prefix sum.
+    // The small arrays sit at the front, so that their places need no width.
+    int* off = reinterpret_cast<int*>(smem);
+    unsigned short* cnt = reinterpret_cast<unsigned short*>(off + ns + 1);
+    double* sb = reinterpret_cast<double*>(smem + ((4 * (ns + 1) + 64 * ns + 15) & ~15));
+    double* sy = sb + rows;
+    double* sv = sy + rows;
+    const bool front = 4ll * (ns + 1) + 64ll * ns + 16ll * rows + 32 <= (long long)dynamic_smem_bytes();
+    __syncthreads();
+    if (!s_start) return;
+    if (front) {
+        for (int s = warp; s < ns; s += MW + 2) {
+            const int r = s * RPS + lane / L, q = lane % L;
+            int my = 0;
+            if (r < rows) {
+                const int len = __ldg(m.rowptr + r0 + r + 1) - __ldg(m.rowptr + r0 + r);
+                my = L == 1 ? len : (len > q ? (len - q + L - 1) / L : 0);
+            }
+            cnt[32 * s + lane] = (unsigned short)my;
+            const int w = (int)__reduce_max_sync(0xffffffffu, (unsigned)my);
+            if (lane == 0) off[s] = w;
+        }
+    }
+    __syncthreads();
+    if (warp == 0 && front) {
+        int base = 0;
+        for (int s0 = 0; s0 < ns; s0 += 32) {
+            const int w = s0 + lane < ns ? off[s0 + lane] : 0;
+            int inc = w;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += t;
+            }
+            if (s0 + lane < ns) off[s0 + lane] = base + inc - w;
+            base += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        if (lane == 0) {
+            off[ns] = base;
+            s_words = base * 32;
+        }
+    }
+    __syncthreads();
+    // the rows must fit the dynamic shared memory of the launch
+    if (!front || resident_bytes(s_words, rows, ns) > (long long)dynamic_smem_bytes()) {
+        if (tid == 0) atomicOr(&ctl->status, ST_CONFIG);
+        return;
+    }
+    int* sc = reinterpret_cast<int*>(sv + s_words);
+    const int xb0 = s_xb;
+    for (int s = warp; s < ns; s += MW + 2) {
+        const int r = s * RPS + lane / L, q = lane % L;
+        if (r < rows) {
+            const int kb = __ldg(m.rowptr + r0 + r) + q, my = cnt[32 * s + lane];
+            double* dv = sv + 32 * off[s] + lane;
+            int* dc = sc + 32 * off[s] + lane;
+            for (int e = 0; e < my; ++e) {
+                dv[32 * e] = __ldg(m.S64 + kb + e * L);
+                dc[32 * e] = __ldg(m.col + kb + e * L);
+            }
+            if (q == 0) {
+                sb[r] = __ldg(m.b + r0 + r);
+                sy[r] = __ldcg(s_x[xb0] + r0 + r);
+            }
+        }
+    }
+    __syncthreads();
+
+    int ksw = max_sweeps;
+    if (!s_dec.test) {
+        const long long rem = s_dec.k_limit - s_dec.k;
+        ksw = (int)(rem < (long long)ksw ? (rem > 0 ? rem : 0) : ksw);
+    }
+    const int active = 32 * (ns < MW ? ns : MW);      // math threads with rows
+    const long long budget = s_budget;
+    unsigned long long arrivals = 0;
+    unsigned long long tr_comp = 0, tr_wait = 0, tr_mark = 0;
+    if (tid == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(tr_mark));
+    // Bounded grid barrier by thread 0: release of the CTA's stores (ordered
+    // before by the CTA barrier), arrival, acquire by the load that sees the
+    // last arrival; the CTA barrier after it extends that to every thread.
+    auto grid_barrier = [&]() {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        tr_comp += t - tr_mark;
+        tr_mark = t;
+        fence_acq_rel_gpu();
+        if (s_skip != (int)blockIdx.x) atomicAdd(&ctl->bar, 1ull);
+        arrivals += gridDim.x;
+        const long long t0 = clock64();
+        int spins = 0;
+        while (ld_acquire_u64(&ctl->bar) < arrivals) {
+            if ((++spins & 63) == 0) {
+                if (ld_volatile_i32(&ctl->status) & ST_TIMEOUT) { s_fail = 1; break; }
+                if (clock64() - t0 > budget) { atomicOr(&ctl->status, ST_TIMEOUT); s_fail = 1; break; }
+            }
+        }
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        tr_wait += t - tr_mark;
+        tr_mark = t;
+    };
+
+    int stop_at = -1;        // sweep whose decision ended the launch
+    int ran = 0;             // sweeps whose barrier has passed
+    for (int s = 0; s < ksw; ++s) {
+        if (warp < MW) {
+            const double* xs = s_x[(xb0 + s) & 3];
+            double* xd = s_x[(xb0 + s + 1) & 3];
+            double ss = 0.0;
+            unsigned long long mx = 0;
+            for (int sl = warp; sl < ns; sl += MW) {
+                const int base = 32 * off[sl] + lane, w = off[sl + 1] - off[sl];
+                const int my = cnt[32 * sl + lane];
+                const int r = sl * RPS + lane / L;
+                const bool lead = r < rows && lane % L == 0;
+                const double* pv = sv + base;
+                const int* pc = sc + base;
+                double acc = lead ? sb[r] : 0.0;
+                for (int o = 0; o < w; o += CH) {
+                    double xv[CH];
+#pragma unroll
+                    for (int u = 0; u < CH; ++u)
+                        if (o + u < my) xv[u] = __ldca(xs + pc[32 * (o + u)]);
+#pragma unroll
+                    for (int u = 0; u < CH; ++u) {
+                        if (o + u >= w) break;
+                        if (o + u < my) acc = __fma_rn(pv[32 * (o + u)], xv[u], acc);
+                    }
+                }
+#pragma unroll
+                for (int d = L / 2; d >= 1; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+                if (lead) {
+                    __stcg(xd + r0 + r, acc);
+                    accumulate_residual(acc, sy[r], ss, mx);
+                    sy[r] = acc;
+                }
+            }
+            if (warp < ns) {
+                s_ss[s & 1][tid] = ss;
+                s_mx[s & 1][tid] = mx;
+            }
+        } else if (warp == MW) {
+            if (s >= 1) publish(s_ss[(s - 1) & 1], s_mx[(s - 1) & 1], active, v.part + ((s - 1) & 1) * v.nslots + blockIdx.x);
+        } else {
+            if (s >= 2) take_decision(s_dec, v.part + (s & 1) * v.nslots, ctl, s - 2, false);
+        }
+        cta_sync<1>();
+        if (s >= 2 && s_dec.done != DONE_RUNNING) { stop_at = s - 2; break; }
+        if (tid == 0) grid_barrier();
+        cta_sync<2>();
+        if (s_fail) break;
+        ++ran;
+    }
+    if (stop_at < 0 && !s_fail && ksw > 0) {
+        // the decisions of the last two sweeps
+        if (warp == MW)
+            publish(s_ss[(ksw - 1) & 1], s_mx[(ksw - 1) & 1], active, v.part + ((ksw - 1) & 1) * v.nslots + blockIdx.x);
+        else if (warp == MW + 1 && ksw >= 2)
+            take_decision(s_dec, v.part + (ksw & 1) * v.nslots, ctl, ksw - 2, false);
+        cta_sync<1>();
+        if (ksw >= 2 && s_dec.done != DONE_RUNNING) {
+            stop_at = ksw - 2;
+        } else {
+            if (tid == 0) grid_barrier();
+            cta_sync<2>();
+            if (!s_fail) {
+                if (warp == MW + 1) take_decision(s_dec, v.part + ((ksw - 1) & 1) * v.nslots, ctl, ksw - 1, true);
+                cta_sync<1>();
+                if (s_dec.done != DONE_RUNNING) stop_at = ksw - 1;
+            }
+        }
+    }
+    if (tid == 0 && v.trace) {
+        atomicAdd(v.trace + 4 * blockIdx.x + 0, tr_comp);
+        atomicAdd(v.trace + 4 * blockIdx.x + 1, tr_wait);
+        atomicAdd(v.trace + 4 * blockIdx.x + 2, (unsigned long long)ran);
+    }
+    if (blockIdx.x == 0 && tid == 0 && ksw > 0) {
+        // x^{k+j} where sweep j's decision stopped the launch, else the last sweep's result
+        const int j = stop_at >= 0 ? stop_at : ran;
+        ctl->k = s_dec.k + j;
+        ctl->xbuf = (xb0 + j) & 3;
+        ctl->evals = s_dec.hist_at + (stop_at >= 0 ? stop_at + 1 : ran);
+        if (stop_at >= 0) ctl->done = s_dec.done;
+        ctl->relres = s_dec.relres;
+        ctl->res2 = s_dec.res2;
+        ctl->resinf = s_dec.resinf;
+        ctl->k_eval = s_dec.k_eval;
+        __threadfence();
+    }
+}
+
+const void* resident_kernel(int lanes)
+{
+    if (lanes == 1) return reinterpret_cast<const void*>(&k_resident<1>);
+    if (lanes == 2) return reinterpret_cast<const void*>(&k_resident<2>);
+    return nullptr;
+}
+
+int resident_threads() { return RT; }
+
+cudaError_t launch_resident(const void* fn, int grid, int smem, const DevMat& m, const DevVec& v, const int* cta_row,
+                            JacCtl* ctl, int max_sweeps, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(RT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[] = {(void*)&m, (void*)&v, (void*)&cta_row, (void*)&ctl, (void*)&max_sweeps};
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+}  // namespace jac
