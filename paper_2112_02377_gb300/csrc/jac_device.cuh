@@ -32,6 +32,7 @@ struct JacCtl {
     unsigned long long bar;   // grid-barrier arrivals of the current launch
     // neighbour-synchronised sweeps (reset with `bar` before every launch):
     unsigned long long dec_ready;  // sweeps of the launch whose grid-wide residual sums are published
+                                   // (resident kernel: sweeps decided | DONE_* of the last << 32)
     unsigned int arrive[4];        // CTAs that finished sweep j, slot j mod 4
     unsigned int ticket;      // last-block detection of the per-sweep launch kernel
     int status;               // ST_* bits
@@ -94,8 +95,8 @@ struct DevMat {
 };
 
 struct DevVec {
-    double* x[4];             // FP64 iterate y = D x: nbuf buffers used in rotation
-    int nbuf;                 // 2 (ping-pong), 3 (neighbour-synchronised sweeps) or 4 (resident kernel)
+    double* x[5];             // FP64 iterate y = D x: nbuf buffers used in rotation
+    int nbuf;                 // 2 (ping-pong), 3 (neighbour-synchronised sweeps) or 5 (resident kernel)
     float* e[2];              // FP32 inner iterate f = D e, ping-pong (mixed)
     float* dlt;               // FP32 residual r of the last P64R pass (mixed)
     Partial* part;            // [2][nslots] per-sweep partial norms
@@ -186,6 +187,16 @@ __device__ __forceinline__ unsigned long long warp_max(unsigned long long v)
     #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = umax64(v, __shfl_down_sync(0xffffffffu, v, o));
     return v;
+}
+
+// As warp_max, in every lane: the high words' maximum, then the low words' among
+// the lanes that hold it.
+__device__ __forceinline__ unsigned long long warp_max_all(unsigned long long v)
+{
+    const unsigned hi = (unsigned)(v >> 32);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)v : 0u);
+    return ((unsigned long long)mh << 32) | ml;
 }
 
 // Residual bookkeeping of one row from its update: r = y' - y = (b - A x)_i.
@@ -404,6 +415,11 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p)
 __device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v)
 {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v)
+{
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 __device__ __forceinline__ int ld_volatile_i32(const int* p)
