@@ -98,11 +98,35 @@ __device__ __forceinline__ void block_sums(double& ss, double& mx, double& bb)
 // Entries staged at a time: a block's 256 rows of up to 7 entries in one
 // round (21.5 KB, eight blocks an SM); longer rows take several rounds.
 constexpr int kCap = 7 * kBlock;
-constexpr int kGather = 8;   // x loads of a row issued together
+constexpr int kGather = 7;   // x loads of a row issued together
 
 __device__ __forceinline__ unsigned shared_addr(const void* p)
 {
     return (unsigned)__cvta_generic_to_shared(p);
+}
+
+// t / d in five FP64 operations where IEEE division takes about twice as many,
+// on a chip whose FP64 pipe bounds the sweep: a single-precision reciprocal of d
+// (its leading bits, moved between the formats with integer operations), one
+// Newton step, and Markstein's quotient correction (Markstein, IBM J. Res. Dev.
+// 34 (1990) 111): q = t r, q + (t - d q) r.  r is good to 2^-44, so the value
+// rounded in the last operation is within 2^-86 of t / d.  Outside exponents
+// that keep every step normal, and for t = 0, the division itself.
+__device__ __forceinline__ double quotient(double t, double d)
+{
+    const unsigned dh = (unsigned)__double2hiint(d), dl = (unsigned)__double2loint(d);
+    const unsigned th = (unsigned)__double2hiint(t);
+    const unsigned de = (dh >> 20) & 0x7ffu, te = (th >> 20) & 0x7ffu;
+    if (de - 923u > 200u || te - 200u > 1600u) return t / d;     // |d| in 2^-100 .. 2^100, |t| in 2^-823 .. 2^777
+    const float f = __uint_as_float((dh & 0x80000000u) | (((dh & 0x7fffffffu) - (896u << 20)) << 3) | (dl >> 29));
+    float rf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+    const unsigned rb = __float_as_uint(rf);
+    const double r0 = __hiloint2double((int)((rb & 0x80000000u) | (((rb & 0x7fffffffu) >> 3) + (896u << 20))),
+                                       (int)(rb << 29));
+    const double r = __fma_rn(__fma_rn(-d, r0, 1.0), r0, r0);
+    const double q = __dmul_rn(t, r);
+    return __fma_rn(__fma_rn(-d, q, t), r, q);
 }
 
 // One sweep on a CSR matrix that stores its diagonal, one thread per row:
@@ -122,6 +146,14 @@ __device__ __forceinline__ unsigned shared_addr(const void* p)
 // before griddepcontrol.wait: the launches of a call depend on one another
 // programmatically, so a sweep's matrix is already arriving while the sweep
 // before it drains.
+//
+// Bound by the FP64 pipe (six FMAs, a subtraction and the quotient's five
+// operations per 7-point row) with the 104 bytes a row moves close behind: about
+// 60 us each for 3,374,850 rows, which take 91 us a sweep (105 with IEEE
+// division; 3,050 before rows were staged); 110,544 rows 7.2 us, 1,188 rows
+// 3.3 us.  Five blocks an SM (48 registers) measured best, seven gathers
+// together as good as eight; a block that copies its next tile while it sums one
+// (two buffers, four blocks) took 105 us.
 template <bool LAST>
 __global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* __restrict__ rowptr,
                                                              const int* __restrict__ col,
@@ -183,7 +215,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* _
         }
     }
     const double t = bi - s;
-    if (i < n) y[i] = t / d;
+    if (i < n) y[i] = quotient(t, d);
     if constexpr (LAST) {
         double ss = 0.0, mx = 0.0, bb = 0.0;
         if (i < n) {

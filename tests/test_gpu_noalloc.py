@@ -1,8 +1,9 @@
 """The allocation-free sweep's staged kernel at the sizes where its blocks and
 rounds end: n around multiples of 256 rows, blocks of more entries than one
 staged round (7 per row), rows longer than a round, the diagonal anywhere in a
-row, arrays with no more than their types' alignment, and a CSR whose rowptr
-starts past zero; against the CPU oracle's sweeps.
+row, arrays with no more than their types' alignment, a CSR whose rowptr
+starts past zero, and the ends of the quotient's fast range; against the CPU
+oracle's sweeps.
 
 Tolerance, from the rounding of one sweep: each side sums len_i terms and
 divides, so x'_i carries at most (len_i + 3) roundings of the row's magnitude
@@ -26,7 +27,8 @@ def _laplace_rows(n):
     return A
 
 
-@pytest.mark.parametrize("name", ["n1", "n255", "n256", "n257", "n513", "fe27", "irregular", "long_row", "offset"])
+@pytest.mark.parametrize("name", ["n1", "n255", "n256", "n257", "n513", "fe27", "irregular", "long_row", "offset", "scale-300",
+                                  "scale-101", "scale99", "scale300", "zeros"])
 def test_noalloc_staged_rounds(name):
     import torch
     if name[0] == "n":
@@ -40,8 +42,14 @@ def test_noalloc_staged_rounds(name):
     else:
         A = W.diffusion7((11, 10, 9), seed=6)
     rng = np.random.default_rng(11)
+    if name.startswith("scale"):                   # diagonals inside and outside the quotient's fast range
+        A.val[:] = A.val * 2.0 ** int(name[5:])
     b, x0 = rng.uniform(-1, 1, A.n), rng.uniform(-1, 1, A.n)
     rp, cl, vl = A.rowptr.copy(), A.col, A.val
+    if name.startswith("scale"):
+        b = b * 2.0 ** int(name[5:])
+    if name == "zeros":                            # rows whose b_i - s_i is zero
+        b[::3], x0[:] = 0.0, 0.0
     shift = 3 if name == "offset" else 0
     if shift:                                      # entries before the first row, and 8 / 4-byte aligned arrays
         rp = rp + shift
