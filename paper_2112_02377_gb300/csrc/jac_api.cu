@@ -52,8 +52,8 @@ struct jac_ctx {
     float* d_S32 = nullptr;
     double* d_b = nullptr;         // b in the new row order (FP64 sweep input)
     double* d_d = nullptr;
-    double* d_x[4] = {nullptr, nullptr, nullptr, nullptr};
-    int nbuf = 2;                  // iterate buffers in rotation (3 with neighbour sync, 4 in the resident kernel)
+    double* d_x[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    int nbuf = 2;                  // iterate buffers in rotation (3 with neighbour sync, 5 in the resident kernel)
     bool resident = false;         // FP64 sweeps run in the resident kernel
     int* d_cta_row = nullptr;      // resident kernel: ctas+1 first rows
     bool ns = false;               // neighbour-synchronised FP64 sweeps
@@ -299,6 +299,7 @@ DevVec devvec(const jac_ctx* c)
     v.x[1] = c->d_x[1];
     v.x[2] = c->d_x[2];
     v.x[3] = c->d_x[3];
+    v.x[4] = c->d_x[4];
     v.nbuf = c->nbuf;
     v.e[0] = c->d_e[0];
     v.e[1] = c->d_e[1];
@@ -574,7 +575,8 @@ void destroy(jac_ctx* c)
     if (c->ev0) cudaEventDestroy(c->ev0);
     if (c->ev1) cudaEventDestroy(c->ev1);
     dfree(c->d_rowptr); dfree(c->d_col); dfree(c->d_S64); dfree(c->d_S32); dfree(c->d_b); dfree(c->d_d);
-    dfree(c->d_x[0]); dfree(c->d_x[1]); dfree(c->d_x[2]); dfree(c->d_x[3]); dfree(c->d_cta_row);
+    dfree(c->d_x[0]); dfree(c->d_x[1]); dfree(c->d_x[2]); dfree(c->d_x[3]); dfree(c->d_x[4]);
+    dfree(c->d_cta_row);
     dfree(c->d_dep_ptr); dfree(c->d_dep); dfree(c->d_done); dfree(c->d_e[0]); dfree(c->d_e[1]); dfree(c->d_dlt);
     dfree(c->d_part); dfree(c->d_ctl); dfree(c->d_hist); dfree(c->d_perm); dfree(c->d_stage); dfree(c->d_stage2);
     dfree(c->d_bmap); dfree(c->d_slot_info);
@@ -928,19 +930,22 @@ static void default_geometry(int lanes, bool mixed, int64_t rows, int* per_sm, i
 
 // Row ranges of the resident kernel's CTAs and the dynamic shared memory of the
 // largest; 0 if a row is too long for it.  It is used wherever it fits: measured
-// on GB300, us per sweep, pipelined / resident: 7-point 8^3 6.8 / 2.7, 32^3 6.9 /
-// 2.9, 48^3 8.4 / 3.7, 64^3 10.7 / 6.0, 70^3 12.0 / 7.1 (74^3 does not fit);
-// 27-point 16^3 7.5 / 2.8, 32^3 8.6 / 4.5, 44^3 11.7 / 7.5 (48^3 does not fit).
+// on GB300, us per sweep, pipelined / resident: 7-point 16^3 7.0 / 2.3, 32^3 6.9 /
+// 2.7, 48^3 8.4 / 3.7, 64^3 10.7 / 5.9, 70^3 12.0 / 7.1 (74^3 does not fit);
+// 27-point 16^3 7.5 / 2.9, 32^3 8.6 / 4.5, 44^3 11.7 / 7.5 (48^3 does not fit).
 static int64_t resident_plan(const ScaledForm& tf, const Plan& plan, int ctas, int lanes,
                              const std::vector<double>* row_cost, std::vector<int32_t>& cut)
 {
     // cheap bound first: entries, b, the iterate and the counts of an even share
     if ((12.0 * tf.rowptr[tf.n] + 18.0 * tf.n) / ctas > 227.0 * 1024) return 0;
     Tiling t;
-    make_tiling(tf, plan, 1 << 30, 1 << 30, ctas, t, row_cost);
-    cut.resize(ctas + 1);
+    // CTA 0 takes the decisions and no rows: sharing its FP64 pipe made its sweeps
+    // 0.35 us longer than the others' (33^3 Q1 replay)
+    const int first = ctas > 1 ? 1 : 0;
+    make_tiling(tf, plan, 1 << 30, 1 << 30, ctas - first, t, row_cost);
+    cut.assign(ctas + 1, 0);
     int64_t most = 0;
-    for (int g = 0; g <= ctas; ++g) cut[g] = t.row0[t.cta0[g]];
+    for (int g = first; g <= ctas; ++g) cut[g] = t.row0[t.cta0[g - first]];
     for (int g = 0; g < ctas; ++g) {
         const int64_t b = resident_smem_bytes(tf.rowptr.data(), cut[g], cut[g + 1], lanes);
         if (b < 0) return 0;
@@ -1043,7 +1048,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
             c->smem = (int)need;
             c->stages = 0;
             c->ntiles = G;
-            c->nbuf = 4;
+            c->nbuf = 5;
             c->h_cta_row0 = cut;
         } else {
             cudaGetLastError();
@@ -1250,8 +1255,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         CK(nullptr, dalloc(&c->d_x[2], n + 16));
     }
     if (c->resident) {
-        CK(nullptr, dalloc(&c->d_x[2], n + 16));
-        CK(nullptr, dalloc(&c->d_x[3], n + 16));
+        for (int q = 2; q < 5; ++q) CK(nullptr, dalloc(&c->d_x[q], n + 16));
         CK(nullptr, dalloc(&c->d_cta_row, (size_t)c->grid + 1));
         CK(nullptr, cudaMemcpy(c->d_cta_row, c->h_cta_row0.data(), (c->grid + 1) * sizeof(int32_t),
                                cudaMemcpyHostToDevice));
@@ -1262,7 +1266,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         CK(nullptr, dalloc(&c->d_e[1], n + 16));
         CK(nullptr, dalloc(&c->d_dlt, n + 16));
     }
-    CK(nullptr, dalloc(&c->d_part, 2 * (size_t)c->nslots + 4 + 2));
+    CK(nullptr, dalloc(&c->d_part, (c->resident ? 4 : 2) * (size_t)c->nslots + 4 + 2));
     if (c->stop == JAC_STOP_LOCAL) {
         std::vector<int32_t> mem_ptr, mem_part, mem_head;
         const Error el = local_row_sets(plan, o, mem_ptr, mem_part, mem_head, c->h_set_id);
@@ -1356,6 +1360,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         add_canary(C, "x[1]", c->d_x[1], nn);
         add_canary(C, "x[2]", c->d_x[2], nn);
         add_canary(C, "x[3]", c->d_x[3], nn);
+        add_canary(C, "x[4]", c->d_x[4], nn);
         add_canary(C, "e[0]", c->d_e[0], nn);
         add_canary(C, "e[1]", c->d_e[1], nn);
         add_canary(C, "r (FP32)", c->d_dlt, nn);

@@ -11,18 +11,21 @@
 // a small system.  It is taken off the chain altogether:
 //   sweep s      the math warps leave each thread's sum of r^2 and max |r| in
 //                shared memory;
-//   sweep s + 1  one spare warp adds them and publishes the CTA's partial sums;
-//   sweep s + 2  another spare warp adds all CTAs' partials (the barrier of
-//                sweep s + 1 made them visible) and takes the decision of sweep s.
-// The iterate rotates through four buffers, so the x^k that a stop returns is
-// still there two sweeps later; counts, results and histories are those of the
-// other kernels.
+//   sweep s + 1  a spare warp adds them and publishes the CTA's partial sums;
+//   sweep s + 2  a spare warp of CTA 0 adds all CTAs' partials (the barrier of
+//                sweep s + 1 made them visible), takes the decision of sweep s and
+//                publishes it as one word;
+//   sweep s + 3  every CTA reads that word before it arrives at the barrier.
+// The iterate rotates through five buffers, so the x^k that a stop returns is
+// still there three sweeps later; counts, results and histories are those of
+// the other kernels.
 //
-// Measured on GB300, 16^3 7-point: 2.75 us a sweep, of them 1.2 us in the grid
+// Measured on GB300, 16^3 7-point: 2.42 us a sweep, of them 1.2 us in the grid
 // barrier (a bare one takes 1.4 us; splitting its counter over several lines or
-// polling differently changes less than 3 %); the pipelined kernel takes 7.0.
-// 64^3: 6.0 us against 10.7, of which 3.4 are the FP64 pipe's.  More sizes at the
-// rule in jac_api.cu (resident_plan).
+// polling differently changes less than 3 %); 2.75 with every CTA taking the
+// decisions itself, 7.0 in the pipelined kernel.  64^3: 5.9 us against 10.7, of
+// which 3.4 are the FP64 pipe's.  More sizes at the rule in jac_api.cu
+// (resident_plan).
 #include <cuda_runtime.h>
 
 #include "jac_device.cuh"
@@ -32,23 +35,38 @@ namespace jac {
 
 namespace {
 
-constexpr int MW = 16;                          // math warps
-constexpr int RT = (MW + 2) * 32;               // threads: math warps, then the two spare warps
 constexpr int CH = 8;                           // entries whose gathers are issued together
+constexpr int NBUF = 5;                         // iterate buffers
+constexpr int NPART = 4;                        // sweeps whose partial sums are kept
+
+// Math warps; two spare warps follow.  (20 with two lanes per row: 27-point 32^3
+// 4.54 -> 4.21 us a sweep, but the 33^3 Q1 replay 3.74 -> 3.94: every idle warp
+// costs the barriers something.)
+constexpr int MW = 16;
+constexpr int RT = (MW + 2) * 32;
+
+// A CTA's sums cost the first spare warp up to 21 FP64 instructions, all on the
+// sub-partition of the warps 0, 4, 8, ...; a slice of short rows costs its warp 8.
+// So the first slices go to the warps of the other three only (7-point 48^3
+// 3.92 -> 3.67 us a sweep, 64^3 6.33 -> 5.92; with two lanes, whose slices cost
+// 16, 27-point 32^3 4.1 -> 4.5: none there).
+template <int L>
+constexpr int uneven_slices() { return L == 1 ? 9 : 0; }
 
 struct ResidentDecision {
     long long k, k_limit, hist_at, hist_cap;    // iterate of the launch's first sweep; limits
     double tol, bnorm, pass;
-    double* hist;                               // CTA 0 only
-    int kind, test, done;
+    double* hist;
+    int kind, test;
     double relres, res2, resinf;
     long long k_eval;
 };
 
-template <int ID>
+// Barrier of the math warps and the first spare warp.
+template <int ID, int THREADS>
 __device__ __forceinline__ void cta_sync()
 {
-    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(RT) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
 }
 
 __device__ void init_decision(ResidentDecision& d, const volatile JacCtl* c)
@@ -59,10 +77,9 @@ __device__ void init_decision(ResidentDecision& d, const volatile JacCtl* c)
     d.hist_cap = c->hist_cap;
     d.tol = c->tol;
     d.bnorm = c->bnorm;
-    d.hist = blockIdx.x == 0 ? c->hist : nullptr;
+    d.hist = c->hist;
     d.kind = c->norm_kind;
     d.test = c->test;
-    d.done = DONE_RUNNING;
     d.relres = c->relres;
     d.res2 = c->res2;
     d.resinf = c->resinf;
@@ -76,15 +93,30 @@ __device__ void init_decision(ResidentDecision& d, const volatile JacCtl* c)
     if (!(d.pass > 1e-280)) d.pass = 1.7976931348623157e308;
 }
 
-// The decision of sweep j of the launch, by one warp, from every CTA's partial sums.
-__device__ void take_decision(ResidentDecision& s, const Partial* part, JacCtl* ctl, int j, bool last)
+// The decision of sweep j of the launch, by one warp, from every CTA's partial
+// sums (in every lane).
+__device__ int take_decision(ResidentDecision& s, const Partial* part, JacCtl* ctl, int j, bool last)
 {
-    double tss;
-    unsigned long long tmx;
-    reduce_partials_warp(part, gridDim.x, tss, tmx);
+    int done = DONE_RUNNING;
+    // five partials of a lane are loaded together (one round trip for 160 CTAs)
+    double tss = 0.0;
+    unsigned long long tmx = 0;
+    for (int i = threadIdx.x & 31; i < (int)gridDim.x; i += 160) {
+        ulonglong2 w[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+            w[u] = i + 32 * u < (int)gridDim.x ? __ldcg(reinterpret_cast<const ulonglong2*>(part + i + 32 * u))
+                                               : make_ulonglong2(0ull, 0ull);
+#pragma unroll
+        for (int u = 0; u < 5; ++u) {
+            tss += __longlong_as_double((long long)w[u].x);
+            tmx = umax64(tmx, w[u].y);
+        }
+    }
+    tss = warp_sum(tss);
+    tmx = warp_max_all(tmx);
     if ((threadIdx.x & 31) == 0) {
         const long long k = s.k + j;
-        int done = DONE_RUNNING;
         const bool bad = !(tss <= 1.7976931348623157e308) || tmx >= KEY_INF;
         const bool near = s.kind == 2 ? !(tss > s.pass) : abs_from_key(tmx) <= s.tol;
         if (last || s.hist || bad || (s.test && (k >= s.k_limit || near))) {
@@ -94,11 +126,11 @@ __device__ void take_decision(ResidentDecision& s, const Partial* part, JacCtl* 
             s.resinf = d.resinf;
             s.k_eval = k;
             done = d.done;
-            if (d.numeric_bad && blockIdx.x == 0) atomicOr(&ctl->status, ST_NUMERIC);
+            if (d.numeric_bad) atomicOr(&ctl->status, ST_NUMERIC);
             if (s.hist && s.hist_at + j < s.hist_cap) s.hist[s.hist_at + j] = d.relres;
         }
-        s.done = done;
     }
+    return __shfl_sync(0xffffffffu, done, 0);
 }
 
 // A CTA's partial sums of one sweep, by one warp: its math threads' sums
@@ -113,7 +145,7 @@ __device__ void publish(const double* ss, const unsigned long long* mx, int acti
         b = umax64(b, mx[i]);
     }
     a = warp_sum(a);
-    b = warp_max(b);
+    b = warp_max_all(b);
     if (lane == 0) {
         __stcg(&slot->ss, a);
         __stcg(&slot->mx, b);
@@ -156,14 +188,15 @@ template <int L>
 __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const int* __restrict__ cta_row, JacCtl* ctl,
                                                     int max_sweeps)
 {
+    constexpr int SYNC = (MW + 1) * 32;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ double s_ss[2][MW * 32];
     __shared__ unsigned long long s_mx[2][MW * 32];
     __shared__ ResidentDecision s_dec;
-    __shared__ int s_start, s_skip, s_xb, s_words;
+    __shared__ int s_start, s_skip, s_xb, s_words, s_stop, s_done;
     __shared__ volatile int s_fail;
     __shared__ long long s_budget;
-    __shared__ double* s_x[4];            // (indexed in shared memory: a local copy would be re-read from L2)
+    __shared__ double* s_x[NBUF];            // (indexed in shared memory: a local copy would be re-read from L2)
     constexpr int RPS = 32 / L;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int r0 = cta_row[blockIdx.x], rows = cta_row[blockIdx.x + 1] - r0;
@@ -176,7 +209,8 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
         s_skip = c->fault_skip_cta;
         s_start = c->done == DONE_RUNNING && c->status == 0;
         s_fail = 0;
-        for (int q = 0; q < 4; ++q) s_x[q] = v.x[q];
+        s_stop = -1;
+        for (int q = 0; q < NBUF; ++q) s_x[q] = v.x[q];
     }
     // ---- slice offsets: widths first (kept in the offsets' place), then their prefix sum.
     // The small arrays sit at the front, so that their places need no width.
@@ -251,7 +285,21 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
         const long long rem = s_dec.k_limit - s_dec.k;
         ksw = (int)(rem < (long long)ksw ? (rem > 0 ? rem : 0) : ksw);
     }
-    const int active = 32 * (ns < MW ? ns : MW);      // math threads with rows
+    // slices of this math warp: one of the first X for the warps of sub-partitions
+    // 1 to 3, then X + warp, X + warp + MW, ...
+    constexpr int X = uneven_slices<L>();
+    const int early = X && (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : X;
+    const bool has_early = warp < MW && early < X && early < ns;
+    // math threads whose sums the spare warp adds: up to the last warp with rows
+    const int nx = ns < X ? ns : X;
+    const int last_early = nx ? ((nx - 1) / 3) * 4 + (nx - 1) % 3 + 1 : -1;
+    const int last_round = ns - X < MW ? ns - X - 1 : MW - 1;
+    const int active = 32 * ((last_early > last_round ? last_early : last_round) + 1);
+    for (int i = tid; i < 2 * MW * 32; i += RT) {
+        s_ss[i / (MW * 32)][i % (MW * 32)] = 0.0;
+        s_mx[i / (MW * 32)][i % (MW * 32)] = 0ull;
+    }
+    __syncthreads();
     const long long budget = s_budget;
     unsigned long long arrivals = 0;
     unsigned long long tr_comp = 0, tr_wait = 0, tr_mark = 0;
@@ -280,15 +328,56 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
         tr_mark = t;
     };
 
-    int stop_at = -1;        // sweep whose decision ended the launch
+    // ================================================= decisions (CTA 0's second spare warp)
+    if (warp == MW + 1) {
+        if (blockIdx.x != 0) return;
+        for (int j = 0; j < ksw; ++j) {
+            // sweep j's partials were published before the barrier of sweep j + 1
+            int ok = 1;
+            if (lane == 0) {
+                const unsigned long long target = (unsigned long long)(j + 2) * gridDim.x;
+                const long long t0 = clock64();
+                while (ld_acquire_u64(&ctl->bar) < target) {
+                    if (s_fail) { ok = 0; break; }
+                    if (clock64() - t0 > budget) { atomicOr(&ctl->status, ST_TIMEOUT); ok = 0; break; }
+                }
+            }
+            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+            const int done = take_decision(s_dec, v.part + (j % NPART) * v.nslots, ctl, j, j + 1 >= ksw);
+            // one word: the sweeps decided, and how the last of them ended
+            if (lane == 0) st_release_u64(&ctl->dec_ready, (unsigned long long)(j + 1) | (unsigned long long)done << 32);
+            if (done != DONE_RUNNING) break;
+        }
+        return;
+    }
+    // The word that decides sweep j, or the final one (by one lane); false on a timeout.
+    auto await_decision = [&](int j, unsigned long long& word) -> bool {
+        const long long t0 = clock64();
+        int spins = 0;
+        for (;;) {
+            word = ld_acquire_u64(&ctl->dec_ready);
+            if ((long long)(word & 0xffffffffull) > j || (word >> 32)) return true;
+            if ((++spins & 63) == 0) {
+                if (ld_volatile_i32(&ctl->status) & ST_TIMEOUT) { s_fail = 1; return false; }
+                if (clock64() - t0 > budget) { atomicOr(&ctl->status, ST_TIMEOUT); s_fail = 1; return false; }
+            }
+        }
+    };
+    auto publish_sweep = [&](int j) {
+        publish(s_ss[j & 1], s_mx[j & 1], active, v.part + (j % NPART) * v.nslots + blockIdx.x);
+    };
+
+    int xs_at = xb0;         // buffer of the iterate that the sweep reads
     int ran = 0;             // sweeps whose barrier has passed
+    bool stopped = false;
     for (int s = 0; s < ksw; ++s) {
+        const int xd_at = xs_at + 1 == NBUF ? 0 : xs_at + 1;
         if (warp < MW) {
-            const double* xs = s_x[(xb0 + s) & 3];
-            double* xd = s_x[(xb0 + s + 1) & 3];
+            const double* xs = s_x[xs_at];
+            double* xd = s_x[xd_at];
             double ss = 0.0;
             unsigned long long mx = 0;
-            for (int sl = warp; sl < ns; sl += MW) {
+            for (int sl = has_early ? early : X + warp; sl < ns; sl = sl < X ? X + warp : sl + MW) {
                 const int base = 32 * off[sl] + lane, w = off[sl + 1] - off[sl];
                 const int my = cnt[32 * sl + lane];
                 const int r = sl * RPS + lane / L;
@@ -315,40 +404,41 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
                     sy[r] = acc;
                 }
             }
-            if (warp < ns) {
+            if (has_early || X + warp < ns) {
                 s_ss[s & 1][tid] = ss;
                 s_mx[s & 1][tid] = mx;
             }
-        } else if (warp == MW) {
-            if (s >= 1) publish(s_ss[(s - 1) & 1], s_mx[(s - 1) & 1], active, v.part + ((s - 1) & 1) * v.nslots + blockIdx.x);
         } else {
-            if (s >= 2) take_decision(s_dec, v.part + (s & 1) * v.nslots, ctl, s - 2, false);
-        }
-        cta_sync<1>();
-        if (s >= 2 && s_dec.done != DONE_RUNNING) { stop_at = s - 2; break; }
-        if (tid == 0) grid_barrier();
-        cta_sync<2>();
-        if (s_fail) break;
-        ++ran;
-    }
-    if (stop_at < 0 && !s_fail && ksw > 0) {
-        // the decisions of the last two sweeps
-        if (warp == MW)
-            publish(s_ss[(ksw - 1) & 1], s_mx[(ksw - 1) & 1], active, v.part + ((ksw - 1) & 1) * v.nslots + blockIdx.x);
-        else if (warp == MW + 1 && ksw >= 2)
-            take_decision(s_dec, v.part + (ksw & 1) * v.nslots, ctl, ksw - 2, false);
-        cta_sync<1>();
-        if (ksw >= 2 && s_dec.done != DONE_RUNNING) {
-            stop_at = ksw - 2;
-        } else {
-            if (tid == 0) grid_barrier();
-            cta_sync<2>();
-            if (!s_fail) {
-                if (warp == MW + 1) take_decision(s_dec, v.part + ((ksw - 1) & 1) * v.nslots, ctl, ksw - 1, true);
-                cta_sync<1>();
-                if (s_dec.done != DONE_RUNNING) stop_at = ksw - 1;
+            if (s >= 1) publish_sweep(s - 1);
+            // every CTA stops in the same sweep: on the decision of sweep s - 3,
+            // although later ones may be known
+            unsigned long long word = 0;
+            if (s >= 3 && lane == 0 && await_decision(s - 3, word) && (word >> 32) &&
+                (int)(word & 0xffffffffull) - 1 == s - 3) {
+                s_stop = s - 3;
+                s_done = (int)(word >> 32);
             }
         }
+        cta_sync<1, SYNC>();
+        if ((stopped = s_stop >= 0)) break;
+        if (tid == 0) grid_barrier();
+        cta_sync<2, SYNC>();
+        if (s_fail) break;
+        ++ran;
+        xs_at = xd_at;
+    }
+    if (!stopped && !s_fail && ksw > 0) {
+        // the decisions of the last sweeps
+        if (warp == MW) publish_sweep(ksw - 1);
+        cta_sync<1, SYNC>();
+        if (tid == 0) grid_barrier();
+        cta_sync<2, SYNC>();
+        unsigned long long word = 0;
+        if (!s_fail && warp == MW && lane == 0 && await_decision(ksw - 1, word) && (word >> 32)) {
+            s_stop = (int)(word & 0xffffffffull) - 1;
+            s_done = (int)(word >> 32);
+        }
+        cta_sync<1, SYNC>();
     }
     if (tid == 0 && v.trace) {
         atomicAdd(v.trace + 4 * blockIdx.x + 0, tr_comp);
@@ -357,11 +447,11 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
     }
     if (blockIdx.x == 0 && tid == 0 && ksw > 0) {
         // x^{k+j} where sweep j's decision stopped the launch, else the last sweep's result
-        const int j = stop_at >= 0 ? stop_at : ran;
+        const int stop_at = s_stop, j = stop_at >= 0 ? stop_at : ran;
         ctl->k = s_dec.k + j;
-        ctl->xbuf = (xb0 + j) & 3;
+        ctl->xbuf = (xb0 + j) % NBUF;
         ctl->evals = s_dec.hist_at + (stop_at >= 0 ? stop_at + 1 : ran);
-        if (stop_at >= 0) ctl->done = s_dec.done;
+        if (stop_at >= 0) ctl->done = s_done;
         ctl->relres = s_dec.relres;
         ctl->res2 = s_dec.res2;
         ctl->resinf = s_dec.resinf;
