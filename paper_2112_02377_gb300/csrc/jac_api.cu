@@ -54,6 +54,7 @@ struct jac_ctx {
     double* d_d = nullptr;
     double* d_x[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     int nbuf = 2;                  // iterate buffers in rotation (3 with neighbour sync, 5 in the resident kernel)
+    bool keep_l2 = false;          // the matrix stays in L2 from sweep to sweep
     bool resident = false;         // FP64 sweeps run in the resident kernel
     int* d_cta_row = nullptr;      // resident kernel: ctas+1 first rows
     bool ns = false;               // neighbour-synchronised FP64 sweeps
@@ -326,6 +327,7 @@ DevTiles devtiles(const jac_ctx* c)
     t.blk = c->d_blk;
     t.lcol = c->d_lcol;
     t.ntiles = c->ntiles;
+    t.keep = c->keep_l2 ? 1 : 0;
     t.emax = c->emax;
     t.xcap = c->xcap;
     t.maxruns = c->maxruns;
@@ -910,6 +912,13 @@ try {
 
 inline int64_t nnz_off_of(const ScaledForm& tf) { return tf.rowptr.empty() ? 0 : tf.rowptr.back(); }
 
+// Whether a sweep's matrix entries are left in L2 for the next one instead of
+// streamed through it evict-first.  Measured on GB300, us per sweep, streamed /
+// left: 7-point FP64 96^3 (63 MB of entries) 19.95 / 19.73, 104^3 (80 MB) 23.4 /
+// 26.0, 120^3 (122 MB) 32.3 / 40.4; mixed 96^3 (42 MB) 10.7 / 10.3, 104^3 (53 MB)
+// 12.9 / 12.2, 112^3 (66 MB) 15.5 / 15.6; 27-point mixed 64^3 (51 MB) 10.7 / 10.3.
+static bool fits_l2(int64_t entries, bool mixed) { return (mixed ? 8.0 : 12.0) * (double)entries <= 64e6; }
+
 // CTAs per SM and pipeline stages (0: the default 4) where the caller leaves
 // both open.  Measured on GB300, us per sweep without calibration:
 //   one lane per row (7-point), 2 against 3 CTAs/SM: a third CTA hides more of
@@ -1184,6 +1193,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         }
         row_cost = &split_cost;
     }
+    c->keep_l2 = fits_l2(nnz_off, o.precision == JAC_MIXED);
     if (c->resident) {
     } else if (c->variant == 2 && !sp) {
         make_tiling(tf, plan, c->rows_per_tile / c->lanes, c->emax, c->grid, tl, row_cost);
@@ -1858,6 +1868,7 @@ try {
     c->K = o.sweeps_per_graph;
     c->variant = 2;
     c->h_sys_off = off;
+    c->keep_l2 = fits_l2(nnz_off, o.precision == JAC_MIXED);
 
     // ---- launch configuration: 7 math warps + producer, 2 CTAs/SM, 4 stages
     cudaDeviceProp prop;

@@ -291,7 +291,7 @@ k_batched(DevMat m, DevVec v, DevTiles t, DevBatch bt, JacCtl* ctl, int max_swee
     // ================================================= producer warp
     if (warp == NW) {
         if (lane == 0) {
-            const uint64_t pol = policy_evict_first();
+            const uint64_t pol = t.keep ? policy_unchanged() : policy_evict_first();
             int cached_sys = -1, cached_mask = 0;
             long long issued = 0;
             for (long long j = 0; j < njobs; ++j) {

@@ -120,6 +120,7 @@ struct DevTiles {
     const int* blk;           // run blocks {xlen, own, nruns, flags} + {src, len, dst, 0} x nruns
     const int* lcol;          // nnz_off tile-local columns (halo kernel)
     int ntiles;
+    int keep;                 // 1: the matrix stays in L2 from sweep to sweep (no evict-first)
     int emax;                 // staged entry cap of a tile
     int xcap;                 // x window capacity (elements)
     int maxruns;              // runs per tile
@@ -388,6 +389,13 @@ __device__ __forceinline__ uint64_t policy_evict_first()
 {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+
+__device__ __forceinline__ uint64_t policy_unchanged()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_unchanged.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
 

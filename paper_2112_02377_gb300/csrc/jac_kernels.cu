@@ -543,7 +543,7 @@ k_persistent(DevMat m, DevVec v, DevTiles t, JacCtl* ctl, int max_sweeps)
     // ================================================= producer warp
     if (warp == NW) {
         if (lane == 0) {
-            const uint64_t pol = policy_evict_first();
+            const uint64_t pol = t.keep ? policy_unchanged() : policy_evict_first();
             long long issued = 0;
             for (long long j = 0; j < njobs; ++j) {
                 const int sidx = (int)(j % STAGES);
