@@ -912,6 +912,21 @@ try {
 
 inline int64_t nnz_off_of(const ScaledForm& tf) { return tf.rowptr.empty() ? 0 : tf.rowptr.back(); }
 
+// Sweep cost estimate of a row by the form that sums it, in the units of
+// default_row_cost (its six entries for a row's own work, fitted to one-lane FP64
+// rows).  Several lanes a row: per-CTA times of 27-point operators, whose boundary
+// rows have 11 to 17 entries instead of 26, put the own work at 19 entries in FP64
+// and 50 in mixed cycles, whose FP32 sweeps are bound by the latency of a row's
+// rounds of gathers and not by its entries (96^3 FP64 57.6 -> 54.1 us a sweep, 61^3
+// mixed 10.0 -> 9.2: the first and last CTAs had a third more rows).  Rows of a
+// substructuring's interface gather from several subdomains: their CTAs took
+// 17 % longer in mixed cycles (131x128x125 in 4x4x4: 22.9 -> 21.6 us).
+static double form_row_cost(int64_t len, int lanes, bool mixed, bool interface_row)
+{
+    if (lanes > 1) return (mixed ? 50.0 : 19.0) + (double)len;
+    return default_row_cost(len) * (interface_row && mixed ? 1.17 : 1.0);
+}
+
 // Whether a sweep's matrix entries are left in L2 for the next one instead of
 // streamed through it evict-first.  Measured on GB300, us per sweep, streamed /
 // left: 7-point FP64 96^3 (63 MB of entries) 19.95 / 19.73, 104^3 (80 MB) 23.4 /
@@ -1183,15 +1198,21 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         c->grid = (int)((n + 255) / 256);
         c->emax = 0;
     }
-    // a split interface layout without calibrated costs: slot rows get their own estimate
-    std::vector<double> split_cost;
-    if (sp && !row_cost) {
-        split_cost.resize(rows);
+    // without calibrated costs: estimates by the kernel's form where the caller
+    // leaves the geometry open; in a split interface layout slot rows get their own
+    std::vector<double> est_cost;
+    const bool by_form = all_auto && o.sync == JAC_SYNC_GRID && o.stop == JAC_STOP_GLOBAL;
+    if (!row_cost && !c->resident && c->variant == 2 && (sp || by_form)) {
+        est_cost.resize(rows);
+        const int64_t ifc = plan.splitting == JAC_SUBSTRUCT && !sp ? plan.part_ptr[plan.nparts() - 1] : rows;
         for (int64_t r = 0; r < rows; ++r) {
             const int64_t len = tf.rowptr[r + 1] - tf.rowptr[r];
-            split_cost[r] = r < sp->n_own ? default_row_cost(len) : slot_row_cost(len);
+            est_cost[r] = sp && r >= sp->n_own
+                              ? slot_row_cost(len)
+                              : sp ? default_row_cost(len)
+                                   : form_row_cost(len, c->lanes, o.precision == JAC_MIXED, r >= ifc);
         }
-        row_cost = &split_cost;
+        row_cost = &est_cost;
     }
     c->keep_l2 = fits_l2(nnz_off, o.precision == JAC_MIXED);
     if (c->resident) {
