@@ -40,7 +40,7 @@ struct jac_ctx {
     // split interface block (jac_setup_local): rows at and after n_own are slot rows
     bool split = false;
     int64_t n_own = 0;
-    long long* d_bmap = nullptr;   // rows: original row whose b starts each kernel row's sum, -1 = none
+    int* d_bmap = nullptr;         // rows: original row whose b starts each kernel row's sum, -1 = none
     unsigned* d_slot_info = nullptr;
     int nrhs = 1;
     int splitting = 0, precision = 0, variant = 2;
@@ -77,7 +77,7 @@ struct jac_ctx {
     JacCtl* h_ctl = nullptr;     // pinned mirrors [2]
     double* d_hist = nullptr;
     int64_t hist_cap = 0;
-    long long* d_perm = nullptr;
+    int* d_perm = nullptr;       // original row of each new row (NULL: the same order)
     double* d_stage = nullptr;   // n*nrhs staging (original order)
     double* d_stage2 = nullptr;  // second staging buffer (adjoint)
     double* d_grad = nullptr;    // nnz (adjoint)
@@ -149,7 +149,6 @@ struct jac_ctx {
     // host-side bookkeeping
     int64_t sweeps_total = 0, outer_last = 0;
     double last_ms = 0.0;
-    std::vector<long long> h_perm;
 };
 
 namespace {
@@ -253,6 +252,10 @@ cudaError_t allow_smem(const void* fn, int bytes)
     return e;
 }
 
+// A caller's vector of doubles as the kernels read it: device memory in place
+// (nothing is kept after the call), host memory through `stage`.
+jac_status on_device(jac_ctx* c, const double* src, int memory, size_t count, double* stage, const double** out);
+
 jac_status copy_to_stage(jac_ctx* c, const double* src, int memory, size_t count, double* stage)
 {
     if (memory == JAC_MEM_DEVICE) {
@@ -263,6 +266,17 @@ jac_status copy_to_stage(jac_ctx* c, const double* src, int memory, size_t count
         return fail(c, JAC_EINVAL, "memory must be JAC_MEM_HOST or JAC_MEM_DEVICE");
     }
     return JAC_OK;
+}
+
+// Device memory that kernels may use in place of a staged copy.
+bool in_place(const double* p, int memory) { return memory == JAC_MEM_DEVICE && ((uintptr_t)p & 7u) == 0; }
+
+jac_status on_device(jac_ctx* c, const double* src, int memory, size_t count, double* stage, const double** out)
+{
+    *out = src;
+    if (!src || in_place(src, memory)) return JAC_OK;
+    *out = stage;
+    return copy_to_stage(c, src, memory, count, stage);
 }
 
 double algorithmic_bytes_fp64(int64_t n, int64_t nnz_off)
@@ -1270,7 +1284,8 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     if (sp) {
         CK(nullptr, dalloc(&c->d_bmap, rows + 16));
         CK(nullptr, dalloc(&c->d_slot_info, sp->slot_info.size() + 16));
-        CK(nullptr, cudaMemcpy(c->d_bmap, sp->bmap.data(), rows * sizeof(long long), cudaMemcpyHostToDevice));
+        const std::vector<int32_t> bmap(sp->bmap.begin(), sp->bmap.end());
+        CK(nullptr, cudaMemcpy(c->d_bmap, bmap.data(), rows * sizeof(int32_t), cudaMemcpyHostToDevice));
         if (!sp->slot_info.empty())
             CK(nullptr, cudaMemcpy(c->d_slot_info, sp->slot_info.data(), sp->slot_info.size() * 4,
                                    cudaMemcpyHostToDevice));
@@ -1316,7 +1331,6 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     }
     if (c->variant >= 2) CK(nullptr, dalloc(&c->d_trace, 4 * (size_t)c->grid));
     CK(nullptr, dalloc(&c->d_ctl, 1));
-    CK(nullptr, dalloc(&c->d_perm, n));
     CK(nullptr, dalloc(&c->d_stage, n + 16));
     CK(nullptr, cudaMallocHost((void**)&c->h_ctl, 2 * sizeof(JacCtl)));
     std::memset(c->h_ctl, 0, 2 * sizeof(JacCtl));
@@ -1365,8 +1379,11 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         }
     }
     CK(nullptr, cudaMemcpy(c->d_d, tf.d.data(), n * 8, cudaMemcpyHostToDevice));
-    c->h_perm.assign(plan.perm.begin(), plan.perm.end());
-    CK(nullptr, cudaMemcpy(c->d_perm, c->h_perm.data(), n * sizeof(long long), cudaMemcpyHostToDevice));
+    if (sp || plan.splitting == JAC_SUBSTRUCT) {   // bands keep the caller's row order
+        const std::vector<int32_t> perm(plan.perm.begin(), plan.perm.end());
+        CK(nullptr, dalloc(&c->d_perm, n));
+        CK(nullptr, cudaMemcpy(c->d_perm, perm.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
+    }
     // original pattern for the adjoint gradient (forward contexts)
     if (pattern) {
         const HostCSR& P = *pattern;
@@ -1401,12 +1418,11 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     }
     // right-hand side and control block
     cudaStream_t sm = stream_of(C);
-    if (b) {
-        st = copy_to_stage(C, b, b_memory, (size_t)n, c->d_stage);
-        if (st != JAC_OK) return fail(nullptr, st, C->err);
-    }
-    CK(nullptr, launch_gather_b(sp ? c->d_bmap : c->d_perm, b ? c->d_stage : nullptr, c->d_b, (int)rows, (int)n,
-                                c->d_ctl, sm));
+    const double* bd = nullptr;
+    st = on_device(C, b, b_memory, (size_t)n, c->d_stage, &bd);
+    if (st != JAC_OK) return fail(nullptr, st, C->err);
+    CK(nullptr, launch_gather_b(sp ? c->d_bmap : c->d_perm, bd, c->d_b, (int)rows, c->d_part, 2 * c->nslots, c->d_ctl,
+                                sm));
     CK(nullptr, launch_reset_iterate(c->d_ctl, sm));
     CK(nullptr, launch_arm(c->d_ctl, 0, 0, o.inner_sweeps, 0, 0, -1.0, o.norm, c->d_hist, c->hist_cap, (long long)o.timeout_cycles,
                      o.fault_skip_cta, sm));
@@ -2028,11 +2044,12 @@ try {
         c->sweeps_total = 0;
         return JAC_OK;
     }
-    if (x) {
-        jac_status st = copy_to_stage(c, x, memory, (size_t)c->n, c->d_stage);
-        if (st != JAC_OK) return st;
-    }
-    CK(c, launch_gather_rows(c->d_perm, x ? c->d_stage : nullptr, c->d_d, c->d_x[0], (int)c->n, 1, s));
+    if (x && memory != JAC_MEM_HOST && memory != JAC_MEM_DEVICE)
+        return fail(c, JAC_EINVAL, "memory must be JAC_MEM_HOST or JAC_MEM_DEVICE");
+    const double* xd = nullptr;
+    const jac_status st = on_device(c, x, memory, (size_t)c->n, c->d_stage, &xd);
+    if (st != JAC_OK) return st;
+    CK(c, launch_gather_rows(c->d_perm, xd, c->d_d, c->d_x[0], (int)c->n, s));
     CK(c, launch_reset_iterate(c->d_ctl, s));
     if (fetch_ctl(c, &c->h_ctl[0]) != JAC_OK) return JAC_ECUDA;
     CK(c, s ? cudaStreamSynchronize(s) : cudaDeviceSynchronize());
@@ -2057,12 +2074,11 @@ try {
         CK(c, s ? cudaStreamSynchronize(s) : cudaDeviceSynchronize());
         return JAC_OK;
     }
-    if (b) {
-        jac_status st = copy_to_stage(c, b, memory, (size_t)c->n, c->d_stage);
-        if (st != JAC_OK) return st;
-    }
-    CK(c, launch_gather_b(c->split ? c->d_bmap : c->d_perm, b ? c->d_stage : nullptr, c->d_b, (int)c->rows,
-                          (int)c->n, c->d_ctl, s));
+    const double* bd = nullptr;
+    const jac_status st = on_device(c, b, memory, (size_t)c->n, c->d_stage, &bd);
+    if (st != JAC_OK) return st;
+    CK(c, launch_gather_b(c->split ? c->d_bmap : c->d_perm, bd, c->d_b, (int)c->rows, c->d_part, 2 * c->nslots, c->d_ctl,
+                          s));
     CK(c, s ? cudaStreamSynchronize(s) : cudaDeviceSynchronize());
     return JAC_OK;
 } catch (...) {
@@ -2279,9 +2295,11 @@ try {
         CK(c, launch_batched_gather_x(c->d_x[0], c->d_x[1], c->d_row_sys, c->d_mask, c->d_kpar, xb, c->n, c->nrhs,
                                       c->d_d, src, s));
     } else {
-        CK(c, launch_scatter_rows(c->d_perm, c->d_x[xb], c->d_d, c->d_stage, (int)c->n, 1, s));
+        if (in_place(x, memory)) src = x;
+        CK(c, launch_scatter_rows(c->d_perm, c->d_x[xb], c->d_d, src, (int)c->n, s));
     }
-    if (memory == JAC_MEM_DEVICE) {
+    if (src == x) {
+    } else if (memory == JAC_MEM_DEVICE) {
         CK(c, cudaMemcpyAsync(x, src, cnt * sizeof(double), cudaMemcpyDeviceToDevice, s));
     } else if (memory == JAC_MEM_HOST) {
         CK(c, cudaMemcpyAsync(x, src, cnt * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2338,15 +2356,26 @@ try {
                                    "built from local matrices)");
     DeviceGuard g(c->device);
     cudaStream_t s = stream_of(c);
-    if (!c->d_stage2) CK(c, dalloc(&c->d_stage2, c->n + 16));
-    if (!c->d_grad) CK(c, dalloc(&c->d_grad, (size_t)c->nnz + 16));
-    jac_status st = copy_to_stage(c, lambda, memory, (size_t)c->n, c->d_stage);
-    if (st != JAC_OK) return st;
-    st = copy_to_stage(c, x, memory, (size_t)c->n, c->d_stage2);
-    if (st != JAC_OK) return st;
-    CK(c, launch_adjoint_grad(c->d_orow, c->d_ocol, c->d_stage, c->d_stage2, c->d_grad, (int)c->n, s));
-    CK(c, cudaMemcpyAsync(dA, c->d_grad, c->nnz * sizeof(double),
-                          memory == JAC_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+    // (dA over lambda or x goes through the staged copies)
+    const uintptr_t g0 = (uintptr_t)dA, g1 = g0 + (size_t)c->nnz * 8;
+    auto apart = [&](const double* p) { return (uintptr_t)p + (size_t)c->n * 8 <= g0 || g1 <= (uintptr_t)p; };
+    const bool direct = in_place(lambda, memory) && in_place(x, memory) && in_place(dA, memory) && apart(lambda) &&
+                        apart(x);
+    if (!direct && !c->d_stage2) CK(c, dalloc(&c->d_stage2, c->n + 16));
+    if (!direct && !c->d_grad) CK(c, dalloc(&c->d_grad, (size_t)c->nnz + 16));
+    const double *ld = lambda, *xd = x;
+    if (!direct) {
+        jac_status st = copy_to_stage(c, lambda, memory, (size_t)c->n, c->d_stage);
+        if (st != JAC_OK) return st;
+        st = copy_to_stage(c, x, memory, (size_t)c->n, c->d_stage2);
+        if (st != JAC_OK) return st;
+        ld = c->d_stage;
+        xd = c->d_stage2;
+    }
+    CK(c, launch_adjoint_grad(c->d_orow, c->d_ocol, ld, xd, direct ? dA : c->d_grad, (int)c->n, s));
+    if (!direct)
+        CK(c, cudaMemcpyAsync(dA, c->d_grad, c->nnz * sizeof(double),
+                              memory == JAC_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     CK(c, s ? cudaStreamSynchronize(s) : cudaDeviceSynchronize());
     return JAC_OK;
 } catch (...) {

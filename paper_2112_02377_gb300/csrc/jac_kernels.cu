@@ -1624,54 +1624,80 @@ const void* halo_kernel(int stages, bool mixed)
 // Small kernels: permutation in/out, right-hand side, control block, adjoint.
 // =========================================================================
 
-// dst[r*nrhs + c] = src[perm[r]*nrhs + c] (src may be NULL = zero)
 // x (caller's row order) -> iterate y_r = a_rr x_perm(r) in the new order
-// (d == nullptr: no scaling; src == nullptr: zero).
-__global__ void k_gather_rows(const long long* __restrict__ perm, const double* __restrict__ src,
-                              const double* __restrict__ d, double* __restrict__ dst, int n, int nrhs)
-{
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n * nrhs) return;
-    const int r = (int)(idx / nrhs), c = (int)(idx - (long long)r * nrhs);
-    const double v = src ? src[perm[r] * nrhs + c] : 0.0;
-    dst[idx] = d ? __dmul_rn(d[r], v) : v;
-}
-
-// iterate y (new order) -> x_perm(r) = y_r / a_rr in the caller's order
-// (IEEE division; d == nullptr: no scaling).
-__global__ void k_scatter_rows(const long long* __restrict__ perm, const double* __restrict__ src,
-                               const double* __restrict__ d, double* __restrict__ dst, int n, int nrhs)
-{
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n * nrhs) return;
-    const int r = (int)(idx / nrhs), c = (int)(idx - (long long)r * nrhs);
-    dst[perm[r] * nrhs + c] = d ? __ddiv_rn(src[idx], d[r]) : src[idx];
-}
-
-// The right-hand side in the new row order: b'_r = b_perm(r) (zero if b is NULL).
-__global__ void k_gather_b(const long long* __restrict__ perm, const double* __restrict__ b, double* __restrict__ out,
-                           int n)
+// (perm == nullptr: the same order; src == nullptr: zero).
+__global__ void k_gather_rows(const int* __restrict__ perm, const double* __restrict__ src,
+                              const double* __restrict__ d, double* __restrict__ dst, int n)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    const long long i = perm[r];
-    out[r] = (b && i >= 0) ? b[i] : 0.0;
+    dst[r] = __dmul_rn(d[r], src ? src[perm ? perm[r] : r] : 0.0);
 }
 
-// ||b||_2 with a fixed reduction order (one CTA of 1024 threads).
-__global__ void __launch_bounds__(1024) k_bnorm(const double* __restrict__ b, long long n, JacCtl* ctl)
+// iterate y (new order) -> x_perm(r) = y_r / a_rr in the caller's order (IEEE division).
+__global__ void k_scatter_rows(const int* __restrict__ perm, const double* __restrict__ src,
+                               const double* __restrict__ d, double* __restrict__ dst, int n)
 {
-    __shared__ double s[32];
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n) return;
+    dst[perm ? perm[r] : r] = __ddiv_rn(src[r], d[r]);
+}
+
+// The right-hand side in the new row order, b'_r = b_perm(r) (zero where perm(r) < 0
+// or b is NULL), and ||b||_2 from the values as they pass: each block's sum in
+// its threads' and a tree's fixed order, the blocks' sums added by the last
+// block to finish.  (A kernel of one block for the norm took 380 us for two
+// million rows, the rest of the call 40.)  The number of blocks depends on the
+// context only, so the norm is the same in every call.
+constexpr int GB_UNROLL = 4;
+__global__ void __launch_bounds__(256) k_gather_b(const int* __restrict__ perm, const double* __restrict__ b,
+                                                  double* __restrict__ out, int n, Partial* part, JacCtl* ctl)
+{
+    __shared__ double s_w[8];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, step = gridDim.x * 256;
     double acc = 0.0;
-    if (b)
-        for (long long i = threadIdx.x; i < n; i += 1024) acc = __fma_rn(b[i], b[i], acc);
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    for (long long r0 = (long long)blockIdx.x * 256 + tid; r0 < n; r0 += (long long)GB_UNROLL * step) {
+        int at[GB_UNROLL];
+        double v[GB_UNROLL];
+#pragma unroll
+        for (int u = 0; u < GB_UNROLL; ++u) {
+            const long long r = r0 + (long long)u * step;
+            at[u] = r < n && b ? (perm ? perm[r] : (int)r) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < GB_UNROLL; ++u) v[u] = at[u] >= 0 ? b[at[u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < GB_UNROLL; ++u) {
+            const long long r = r0 + (long long)u * step;
+            if (r < n) out[r] = v[u];
+            acc = __fma_rn(v[u], v[u], acc);
+        }
+    }
+    auto block_sum = [&](double a) {
+        a = warp_sum(a);
+        if ((tid & 31) == 0) s_w[tid >> 5] = a;
+        __syncthreads();
         double t = 0.0;
-        for (int w = 0; w < 32; ++w) t += s[w];
-        ctl->bnorm = sqrt(t);
+        if (tid == 0)
+            for (int w = 0; w < 8; ++w) t += s_w[w];
+        return t;
+    };
+    const double t = block_sum(acc);
+    if (tid == 0) {
+        part[blockIdx.x].ss = t;
+        __threadfence();
+        s_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    acc = 0.0;
+    for (int q = tid; q < (int)gridDim.x; q += 256) acc += __ldcg(&part[q].ss);
+    const double total = block_sum(acc);
+    if (tid == 0) {
+        ctl->bnorm = sqrt(total);
+        ctl->ticket = 0;
     }
 }
 
@@ -1845,27 +1871,23 @@ cudaError_t launch_persistent(const void* fn, int grid, int threads, int smem, c
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-cudaError_t launch_gather_rows(const long long* perm, const double* src, const double* d, double* dst, int n,
-                               int nrhs, cudaStream_t s)
+cudaError_t launch_gather_rows(const int* perm, const double* src, const double* d, double* dst, int n, cudaStream_t s)
 {
-    const long long tot = (long long)n * nrhs;
-    k_gather_rows<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(perm, src, d, dst, n, nrhs);
+    k_gather_rows<<<(n + 255) / 256, 256, 0, s>>>(perm, src, d, dst, n);
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_rows(const long long* perm, const double* src, const double* d, double* dst, int n,
-                                int nrhs, cudaStream_t s)
+cudaError_t launch_scatter_rows(const int* perm, const double* src, const double* d, double* dst, int n, cudaStream_t s)
 {
-    const long long tot = (long long)n * nrhs;
-    k_scatter_rows<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(perm, src, d, dst, n, nrhs);
+    k_scatter_rows<<<(n + 255) / 256, 256, 0, s>>>(perm, src, d, dst, n);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather_b(const long long* perm, const double* b, double* out, int nout, int nb, JacCtl* ctl,
+cudaError_t launch_gather_b(const int* perm, const double* b, double* out, int n, Partial* part, int nparts, JacCtl* ctl,
                             cudaStream_t s)
 {
-    k_gather_b<<<(nout + 255) / 256, 256, 0, s>>>(perm, b, out, nout);
-    k_bnorm<<<1, 1024, 0, s>>>(b, nb, ctl);
+    const int blocks = (n + 255) / 256;
+    k_gather_b<<<blocks < nparts ? blocks : nparts, 256, 0, s>>>(perm, b, out, n, part, ctl);
     return cudaGetLastError();
 }
 

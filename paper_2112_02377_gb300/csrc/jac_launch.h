@@ -29,13 +29,12 @@ int halo_smem_bytes(int rows, int emax, int xcap, int ntcap, int blkcap, int sta
 cudaError_t launch_persistent(const void* fn, int grid, int threads, int smem, const DevMat& m, const DevVec& v,
                               const DevTiles& t, JacCtl* ctl, int max_sweeps, cudaStream_t s);
 
-// x <-> iterate y = D x conversions (d == nullptr: plain permuted copy)
-cudaError_t launch_gather_rows(const long long* perm, const double* src, const double* d, double* dst, int n,
-                               int nrhs, cudaStream_t s);
-cudaError_t launch_scatter_rows(const long long* perm, const double* src, const double* d, double* dst, int n,
-                                int nrhs, cudaStream_t s);
-// out[r] = b[perm[r]] (0 where perm[r] < 0), r < nout; ||b||_2 over the nb entries of b.
-cudaError_t launch_gather_b(const long long* perm, const double* b, double* out, int nout, int nb, JacCtl* ctl,
+// x <-> iterate y = D x conversions (perm == nullptr: the same row order)
+cudaError_t launch_gather_rows(const int* perm, const double* src, const double* d, double* dst, int n, cudaStream_t s);
+cudaError_t launch_scatter_rows(const int* perm, const double* src, const double* d, double* dst, int n, cudaStream_t s);
+// out[r] = b[perm[r]] (0 where perm[r] < 0 or b is NULL), r < n, and their 2-norm
+// (part: scratch of nparts partial sums).
+cudaError_t launch_gather_b(const int* perm, const double* b, double* out, int n, Partial* part, int nparts, JacCtl* ctl,
                             cudaStream_t s);
 cudaError_t launch_arm(JacCtl* ctl, int test, int mixed, int inner, long long k_limit, long long k_delta,
                        double tol, int norm_kind, double* hist, long long hist_cap, long long timeout, int skip,
