@@ -472,11 +472,22 @@ k_persistent(DevMat m, DevVec v, DevTiles t, JacCtl* ctl, int max_sweeps)
     __shared__ volatile int s_stop;
     __shared__ double s_relres, s_res2, s_resinf;
     __shared__ int s_locpart;
-    __shared__ double s_locval;
+    __shared__ double s_locval, s_pass, s_tol;
+    __shared__ int s_quick;   // decisions without decide(): 2 by the sum, 1 by the maximum, 0 never
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         const volatile JacCtl* c = ctl;
+        {
+            // A sum of squares above s_pass fails the 2-norm test whatever decide()
+            // rounds (the margin covers its roundings and ours); where the product
+            // is too small to carry the margin, decide() is always asked.
+            const double bn = c->bnorm, tl = c->tol, vb = bn > 0.0 ? tl * bn : tl;
+            const double ps = vb * vb * (1.0 + 1e-12);
+            s_pass = ps > 1e-280 ? ps : 1.7976931348623157e308;
+            s_tol = tl;
+            s_quick = c->hist ? 0 : c->norm_kind == 2 ? 2 : 1;
+        }
         s_k = c->k;
         s_klim = c->k_limit;
         s_evals = c->evals;
@@ -950,8 +961,10 @@ k_persistent(DevMat m, DevVec v, DevTiles t, JacCtl* ctl, int max_sweeps)
         }
         // ---- publish partial norms, grid barrier
         if (norm_ph) {
-            const double ws = warp_sum(ss);
-            const unsigned long long wm = warp_max(mx);
+            // a warp without residuals skips the FP64 adds (64 cycles each)
+            const bool any = __any_sync(0xffffffffu, __double_as_longlong(ss) != 0);
+            const double ws = any ? warp_sum(ss) : 0.0;
+            const unsigned long long wm = warp_max_all(mx);
             if (lane == 0) { s_wss[warp] = ws; s_wmx[warp] = wm; }
         }
         if constexpr (ASYNC) {
@@ -1036,17 +1049,23 @@ k_persistent(DevMat m, DevVec v, DevTiles t, JacCtl* ctl, int max_sweeps)
             continue;
         }
         consumer_sync<CT>();
+        double cta_b = 0.0;             // the CTA's sums: a fixed tree over the warps'
+        unsigned long long cta_m = 0;
+        if (norm_ph && warp == 0) {
+            cta_b = lane < NW ? s_wss[lane] : 0.0;
+            cta_m = lane < NW ? s_wmx[lane] : 0ull;
+#pragma unroll
+            for (int o = NW > 8 ? 8 : 4; o > 0; o >>= 1) cta_b += __shfl_xor_sync(0xffffffffu, cta_b, o);
+            cta_m = warp_max_all(cta_m);
+        }
         if (tid == 0) {
             const unsigned long long tb_ = global_ns();
             tr_comp += tb_ - tr_mark;
             tr_mark = tb_;
             if (norm_ph) {
-                double b = 0.0;
-                unsigned long long bm = 0;
-                for (int w = 0; w < NW; ++w) { b += s_wss[w]; bm = umax64(bm, s_wmx[w]); }
                 Partial* slot = v.part + (sw & 1) * v.nslots + blockIdx.x;
-                __stcg(&slot->ss, b);
-                __stcg(&slot->mx, bm);
+                __stcg(&slot->ss, cta_b);
+                __stcg(&slot->mx, cta_m);
             }
             // release: this CTA's stores (ordered before by the CTA barrier) and
             // its partial sums; acquire: the polling load that sees the last
@@ -1055,10 +1074,12 @@ k_persistent(DevMat m, DevVec v, DevTiles t, JacCtl* ctl, int max_sweeps)
             if (!(s_skip == (int)blockIdx.x)) atomicAdd(&ctl->bar, 1ull);
             const unsigned long long target = (unsigned long long)(nbar + 1) * gridDim.x;
             const long long t0 = clock64();
+            int spins = 0;
             while (ld_acquire_u64(&ctl->bar) < target) {
-                if (ld_volatile_i32(&ctl->status) & ST_TIMEOUT) { s_fail = 1; break; }
-                if (clock64() - t0 > budget) { atomicOr(&ctl->status, ST_TIMEOUT); s_fail = 1; break; }
-                __nanosleep(32);
+                if ((++spins & 63) == 0) {
+                    if (ld_volatile_i32(&ctl->status) & ST_TIMEOUT) { s_fail = 1; break; }
+                    if (clock64() - t0 > budget) { atomicOr(&ctl->status, ST_TIMEOUT); s_fail = 1; break; }
+                }
             }
             {
                 const unsigned long long tc_ = global_ns();
@@ -1078,7 +1099,15 @@ k_persistent(DevMat m, DevVec v, DevTiles t, JacCtl* ctl, int max_sweeps)
                 unsigned long long lk = ~0ull;
                 int lp = -1;
                 if constexpr (LOC) local_sets_min(lslot, v.nloc, lk, lp);
-                if (lane == 0) {
+                // Most sweeps are decided without decide()'s square root and division
+                // (500 cycles each on this FP64 pipe, between the barrier and the next
+                // sweep): the values they give are those of the launch's last sweep.
+                bool far = s_quick == 2 ? tss > s_pass : abs_from_key(tmx) > s_tol;
+                if constexpr (LOC) far = far && !(lp >= 0 && lk <= KEY_INF && abs_from_key(lk) <= s_tol);
+                if (lane == 0 && s_quick && sw + 1 < ksw && tmx < KEY_INF && tss <= 1.7976931348623157e308 &&
+                    (!s_test || (far && k < s_klim))) {
+                    s_dec_done = DONE_RUNNING;
+                } else if (lane == 0) {
                     const Decision d = decide(s_test, ctl->tol, s_klim, ctl->norm_kind, ctl->bnorm, tss, tmx, k);
                     s_relres = d.relres;
                     s_res2 = d.res2;
