@@ -346,7 +346,12 @@ try {
             if (g_slots[q].addr && g_slots[q].ctx_id == id) scratch = g_slots[q].addr;
         if (!scratch) {
             void* p = nullptr;
+            // (and both kernels, which lazy loading would otherwise load at the first
+            // call that launches each)
+            cudaFuncAttributes fa;
             e = cudaGetSymbolAddress(&p, g_scratch);
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_noalloc_sweep<false>);
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_noalloc_sweep<true>);
             if (e != cudaSuccess)
                 return fail(JAC_ECUDA, std::string("jac_sweep_noalloc: cudaGetSymbolAddress: ") + cudaGetErrorString(e));
             scratch = static_cast<unsigned char*>(p);
