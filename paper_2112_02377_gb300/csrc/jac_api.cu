@@ -103,7 +103,7 @@ struct jac_ctx {
     int* d_mem_ptr = nullptr;             // rows+1: each row's local sets ...
     int* d_mem_part = nullptr;            // ... as dense set numbers
     int* d_mem_head = nullptr;            // rows: first set | (number of sets << 24)
-    unsigned long long* d_loc = nullptr;  // [3][nloc] per-set maxima of |r| (order keys)
+    unsigned long long* d_loc = nullptr;  // [loc_slots][nloc] per-set maxima of |r| (order keys)
     int nloc = 0;
     std::vector<int32_t> h_set_id;        // partition number of each dense set
     const void* pfn64 = nullptr;
@@ -388,6 +388,9 @@ int mixed_cycles_per_step(const jac_ctx* c)
 // a sweep: its steps have at least 512 sweeps.
 int sweeps_per_step(const jac_ctx* c) { return c->resident ? std::max(c->K, 512) : c->K; }
 
+// Sweeps whose per-set maxima are kept (local stopping).
+int loc_slots(const jac_ctx* c) { return c->resident ? 4 : 3; }
+
 // Enqueue one "graph step": K sweeps (FP64) or one refinement cycle block (mixed).
 jac_status enqueue_step(jac_ctx* c, bool mixed)
 {
@@ -411,6 +414,8 @@ jac_status enqueue_step(jac_ctx* c, bool mixed)
     }
     if (c->resident) {
         CK(c, launch_reset_bar(c->d_ctl, s));
+        // (a launch that stopped leaves the maxima of the sweeps after the stop)
+        if (c->d_loc) CK(c, cudaMemsetAsync(c->d_loc, 0, loc_slots(c) * sizeof(unsigned long long) * c->nloc, s));
         CK(c, launch_resident(c->pfn64, c->grid, c->smem, devmat(c), devvec(c), c->d_cta_row, c->d_ctl,
                               sweeps_per_step(c), s));
         return JAC_OK;
@@ -567,7 +572,8 @@ jac_status arm(jac_ctx* c, int test, int mixed, long long k_limit, long long k_d
 {
     if (c->d_trace)
         CK(c, cudaMemsetAsync(c->d_trace, 0, 4 * sizeof(unsigned long long) * c->grid, stream_of(c)));
-    if (c->d_loc) CK(c, cudaMemsetAsync(c->d_loc, 0, 3 * sizeof(unsigned long long) * c->nloc, stream_of(c)));
+    if (c->d_loc)
+        CK(c, cudaMemsetAsync(c->d_loc, 0, loc_slots(c) * sizeof(unsigned long long) * c->nloc, stream_of(c)));
     CK(c, launch_arm(c->d_ctl, test, mixed, c->o.inner_sweeps, k_limit, k_delta, tol, c->o.norm, c->d_hist, c->hist_cap,
                      (long long)c->o.timeout_cycles, c->o.fault_skip_cta, stream_of(c)));
     return JAC_OK;
@@ -1067,14 +1073,15 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         c->stages = stages;
     // ---- the resident kernel, where the caller leaves the geometry open and the matrix fits
     bool all_auto = o.variant == 0 && !o.tile_rows && !o.ctas_per_sm && !o.stages;
-    if (all_auto && !sp && o.precision == JAC_FP64 && o.sync == JAC_SYNC_GRID && o.stop == JAC_STOP_GLOBAL &&
-        resident_kernel(c->lanes)) {
+    const bool local_stop = o.stop == JAC_STOP_LOCAL;
+    if (all_auto && !sp && o.precision == JAC_FP64 && o.sync == JAC_SYNC_GRID &&
+        resident_kernel(c->lanes, local_stop)) {
         const int G = prop.multiProcessorCount;
         std::vector<int32_t> cut;
         const int64_t need = resident_plan(tf, plan, G, c->lanes, row_cost, cut);
         int coop = 0, fits = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        const void* fn = resident_kernel(c->lanes);
+        const void* fn = resident_kernel(c->lanes, local_stop);
         if (need > 0 && need <= (int64_t)prop.sharedMemPerBlockOptin && coop &&
             allow_smem(fn, (int)need) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, fn, resident_threads(), (size_t)need) == cudaSuccess &&
@@ -1323,11 +1330,11 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         CK(nullptr, dalloc(&c->d_mem_head, mem_head.size() + 1));
         if (!mem_head.empty())
             CK(nullptr, cudaMemcpy(c->d_mem_head, mem_head.data(), mem_head.size() * 4, cudaMemcpyHostToDevice));
-        CK(nullptr, dalloc(&c->d_loc, 3 * (size_t)c->nloc));
+        CK(nullptr, dalloc(&c->d_loc, loc_slots(c.get()) * (size_t)c->nloc));
         CK(nullptr, cudaMemcpy(c->d_mem_ptr, mem_ptr.data(), mem_ptr.size() * 4, cudaMemcpyHostToDevice));
         if (!mem_part.empty())
             CK(nullptr, cudaMemcpy(c->d_mem_part, mem_part.data(), mem_part.size() * 4, cudaMemcpyHostToDevice));
-        CK(nullptr, cudaMemset(c->d_loc, 0, 3 * sizeof(unsigned long long) * c->nloc));
+        CK(nullptr, cudaMemset(c->d_loc, 0, loc_slots(c.get()) * sizeof(unsigned long long) * c->nloc));
     }
     if (c->variant >= 2) CK(nullptr, dalloc(&c->d_trace, 4 * (size_t)c->grid));
     CK(nullptr, dalloc(&c->d_ctl, 1));
@@ -1651,7 +1658,7 @@ try {
     // 2 CTAs/SM and 2 large stages that hold whole tiles of 256/L rows.
     std::vector<Geometry> cand;
     // (FP64 systems that fit the chip's shared memory: what an open geometry gives, the resident kernel)
-    if (o.precision == JAC_FP64 && !async && !local_stop && resident_kernel(la) && !o.stages &&
+    if (o.precision == JAC_FP64 && !async && resident_kernel(la, local_stop) && !o.stages &&
         prep.tf.rowptr[prep.tf.n] <= 3000000)
         cand.push_back({0, 0, 0, 0});
     if (la >= 2 && !async) cand.push_back({2, 256, 2, 0, JAC_SYNC_GRID, 2});

@@ -104,7 +104,8 @@ struct DevVec {
     int nslots;
     unsigned long long* trace;  // [ctas][4]: compute ns, barrier-wait ns, sweeps, 0 (persistent kernels)
     // stopping on local convergence: [3][nloc] per-set max abs_key(r_i); the
-    // residual of iterate k goes to slot k mod 3
+    // residual of iterate k goes to slot k mod 3 (resident kernel: [4][nloc], by
+    // the launch's sweep)
     unsigned long long* loc;
     int nloc;
 };

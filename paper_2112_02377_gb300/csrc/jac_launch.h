@@ -19,7 +19,7 @@ int persistent_threads(int rows);
 // Resident kernel (one CTA per SM, matrix in shared memory): lanes per row 1 or
 // 2, else nullptr; cta_row: grid+1 first rows.  resident_smem_bytes: what rows
 // [r0, r1) need (negative: a row too long).
-const void* resident_kernel(int lanes);
+const void* resident_kernel(int lanes, bool local_stop);
 int resident_threads();
 long long resident_smem_bytes(const int* rowptr, int r0, int r1, int lanes);
 cudaError_t launch_resident(const void* fn, int grid, int smem, const DevMat& m, const DevVec& v, const int* cta_row,

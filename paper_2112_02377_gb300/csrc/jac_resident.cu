@@ -60,6 +60,8 @@ struct ResidentDecision {
     int kind, test;
     double relres, res2, resinf;
     long long k_eval;
+    int loc_part;                               // local stopping: the partition that passed, its value
+    double loc_val;
 };
 
 // Barrier of the math warps and the first spare warp.
@@ -84,6 +86,8 @@ __device__ void init_decision(ResidentDecision& d, const volatile JacCtl* c)
     d.res2 = c->res2;
     d.resinf = c->resinf;
     d.k_eval = c->k_eval;
+    d.loc_part = -1;
+    d.loc_val = 0.0;
     // A sum of squares above this fails the 2-norm test whatever decide()
     // rounds (the margin covers its roundings and ours), so most sweeps are
     // decided without its square root and division.  Where the product is too
@@ -94,10 +98,19 @@ __device__ void init_decision(ResidentDecision& d, const volatile JacCtl* c)
 }
 
 // The decision of sweep j of the launch, by one warp, from every CTA's partial
-// sums (in every lane).
-__device__ int take_decision(ResidentDecision& s, const Partial* part, JacCtl* ctl, int j, bool last)
+// sums (in every lane).  LOC: the first partition whose own rows pass ends the
+// solve too; its maxima are cleared for sweep j + NPART once they have been read.
+template <bool LOC>
+__device__ int take_decision(ResidentDecision& s, const Partial* part, unsigned long long* loc, int nloc, JacCtl* ctl,
+                             int j, bool last)
 {
     int done = DONE_RUNNING;
+    [[maybe_unused]] unsigned long long lk = ~0ull;
+    [[maybe_unused]] int lp = -1;
+    if constexpr (LOC) {
+        local_sets_min(loc, nloc, lk, lp);
+        for (int i = threadIdx.x & 31; i < nloc; i += 32) __stcg(loc + i, 0ull);
+    }
     // five partials of a lane are loaded together (one round trip for 160 CTAs)
     double tss = 0.0;
     unsigned long long tmx = 0;
@@ -118,7 +131,10 @@ __device__ int take_decision(ResidentDecision& s, const Partial* part, JacCtl* c
     if ((threadIdx.x & 31) == 0) {
         const long long k = s.k + j;
         const bool bad = !(tss <= 1.7976931348623157e308) || tmx >= KEY_INF;
-        const bool near = s.kind == 2 ? !(tss > s.pass) : abs_from_key(tmx) <= s.tol;
+        bool near = s.kind == 2 ? !(tss > s.pass) : abs_from_key(tmx) <= s.tol;
+        // (NaN keys never pass)
+        const bool local = LOC && s.test && nloc > 0 && lk <= KEY_INF && abs_from_key(lk) <= s.tol;
+        if constexpr (LOC) near = near || local;
         if (last || s.hist || bad || (s.test && (k >= s.k_limit || near))) {
             const Decision d = decide(s.test, s.tol, s.k_limit, s.kind, s.bnorm, tss, tmx, k);
             s.relres = d.relres;
@@ -126,6 +142,13 @@ __device__ int take_decision(ResidentDecision& s, const Partial* part, JacCtl* c
             s.resinf = d.resinf;
             s.k_eval = k;
             done = d.done;
+            if constexpr (LOC) {
+                if (local && !d.numeric_bad) {
+                    done = DONE_CONVERGED;
+                    s.loc_part = lp;
+                    s.loc_val = abs_from_key(lk);
+                }
+            }
             if (d.numeric_bad) atomicOr(&ctl->status, ST_NUMERIC);
             if (s.hist && s.hist_at + j < s.hist_cap) s.hist[s.hist_at + j] = d.relres;
         }
@@ -184,7 +207,15 @@ long long resident_smem_bytes(const int* rowptr, int r0, int r1, int lanes)
 //
 // Entries are stored slice by slice, entry-major (entry e of lane l at
 // 32 e + l): a warp's reads of S and col are consecutive.
-template <int L>
+//
+// LOC also keeps each partition's max |r| (integer atomics on the sets holding a
+// row, as in the pipelined kernel), in NPART slots of v.loc that start at zero:
+// sweep s raises slot s % NPART, the decision of sweep s reads and clears it, and
+// every CTA has seen that decision before it starts sweep s + NPART.
+// Measured, 33^3 Q1 matrix, us per sweep, pipelined / resident: 8 bands 8.2 / 4.8,
+// 8 boxes 10.3 / 7.0, 64 boxes 12.5 / 7.7 (the global test: 3.7); what it adds is
+// the atomics and, where a warp's rows lie in several boxes, finding the peers.
+template <int L, bool LOC>
 __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const int* __restrict__ cta_row, JacCtl* ctl,
                                                     int max_sweeps)
 {
@@ -343,7 +374,11 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
                 }
             }
             if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-            const int done = take_decision(s_dec, v.part + (j % NPART) * v.nslots, ctl, j, j + 1 >= ksw);
+            __syncwarp();                         // lane 0's acquire, for every lane
+            const int done = take_decision<LOC>(s_dec, v.part + (j % NPART) * v.nslots,
+                                                LOC ? v.loc + (size_t)(j % NPART) * v.nloc : nullptr, v.nloc, ctl, j,
+                                                j + 1 >= ksw);
+            if constexpr (LOC) __syncwarp();      // every lane's cleared maxima before the release
             // one word: the sweeps decided, and how the last of them ended
             if (lane == 0) st_release_u64(&ctl->dec_ready, (unsigned long long)(j + 1) | (unsigned long long)done << 32);
             if (done != DONE_RUNNING) break;
@@ -385,6 +420,8 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
                 const double* pv = sv + base;
                 const int* pc = sc + base;
                 double acc = lead ? sb[r] : 0.0;
+                [[maybe_unused]] int head = -1;
+                if constexpr (LOC) head = lead ? __ldg(m.mem_head + r0 + r) : -1;
                 for (int o = 0; o < w; o += CH) {
                     double xv[CH];
 #pragma unroll
@@ -398,11 +435,16 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
                 }
 #pragma unroll
                 for (int d = L / 2; d >= 1; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+                [[maybe_unused]] unsigned long long key = 0;
                 if (lead) {
                     __stcg(xd + r0 + r, acc);
-                    accumulate_residual(acc, sy[r], ss, mx);
+                    if constexpr (LOC) key = accumulate_residual_key(acc, sy[r], ss, mx);
+                    else accumulate_residual(acc, sy[r], ss, mx);
                     sy[r] = acc;
                 }
+                if constexpr (LOC)
+                    local_sets_update(v.loc + (size_t)(s % NPART) * v.nloc, m.mem_ptr, m.mem_part, lead ? r0 + r : -1,
+                                      head, key);
             }
             if (has_early || X + warp < ns) {
                 s_ss[s & 1][tid] = ss;
@@ -456,14 +498,22 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
         ctl->res2 = s_dec.res2;
         ctl->resinf = s_dec.resinf;
         ctl->k_eval = s_dec.k_eval;
+        if (LOC && s_dec.loc_part >= 0) {
+            ctl->loc_part = s_dec.loc_part;
+            ctl->loc_val = s_dec.loc_val;
+        }
         __threadfence();
     }
 }
 
-const void* resident_kernel(int lanes)
+const void* resident_kernel(int lanes, bool local_stop)
 {
-    if (lanes == 1) return reinterpret_cast<const void*>(&k_resident<1>);
-    if (lanes == 2) return reinterpret_cast<const void*>(&k_resident<2>);
+    if (lanes == 1)
+        return local_stop ? reinterpret_cast<const void*>(&k_resident<1, true>)
+                          : reinterpret_cast<const void*>(&k_resident<1, false>);
+    if (lanes == 2)
+        return local_stop ? reinterpret_cast<const void*>(&k_resident<2, true>)
+                          : reinterpret_cast<const void*>(&k_resident<2, false>);
     return nullptr;
 }
 

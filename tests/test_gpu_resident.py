@@ -90,6 +90,44 @@ def test_resident_solves_stop_at_the_same_sweep(name, split, norm, lanes):
             _same(a, p, A.n)
 
 
+@pytest.mark.parametrize("name,split,parts,lanes", [("line33", "bandrow", 33, 0), ("lap", "bandrow_nnz", 200, 0),
+                                                    ("lap", "substruct", (3, 3, 2), 2), ("q1", "substruct", (2, 2, 2), 0),
+                                                    ("diff", "bandrow", 1, 1), ("fe", "bandrow", 64, 0)])
+def test_resident_local_stop_is_the_pipelined_one(name, split, parts, lanes):
+    """Stopping on local convergence (integer maxima: nothing here may differ)."""
+    A = _matrix(name)
+    b = np.random.default_rng(6).uniform(-1, 1, A.n)
+    kw = dict(subdomains=parts) if split == "substruct" else dict(nparts=parts)
+    a, p = _pair(A, b, split, lanes_per_row=lanes, norm=0, stop=J.JAC_STOP_LOCAL, history=4096, **kw)
+    zero_part = np.where(np.arange(A.n) < A.n // 2, b, 0.0)     # a partition that passes at once, where there are several
+
+    def check(tol, maxit):
+        ka, kp = a.solve(tol, maxit), p.solve(tol, maxit)
+        assert ka == kp
+        _same(a, p, A.n)
+        sa, sp = a.stats(), p.stats()
+        assert sa["stop_part"] == sp["stop_part"] and sa["stop_local"] == sp["stop_local"]
+        assert np.array_equal(a.history(), p.history())
+        return ka[2]
+
+    with a, p:
+        assert a.stats()["ctas_per_sm"] == 1
+        for tol in (0.5, 1e-2, 1e-5, 1e-9):
+            a.set_x(), p.set_x()
+            assert check(tol, 20000) == J.JAC_OK
+            assert check(tol, 20000) == J.JAC_OK    # the returned iterate passes again
+            assert check(tol / 2, 20000) == J.JAC_OK    # and the solve goes on from it
+        for maxit in (0, 1, 2, 3, 513):
+            a.set_x(), p.set_x()
+            assert check(0.0, maxit) == J.JAC_ENOTCONV or maxit > 3     # (a residual may become exactly 0)
+        a.set_b(zero_part), p.set_b(zero_part)
+        a.set_x(), p.set_x()
+        assert check(1e-5, 20000) == J.JAC_OK
+        assert a.sweep(7) == p.sweep(7)             # sweeps without a test raise the maxima too
+        a.set_x(), p.set_x()
+        assert check(1e-7, 20000) == J.JAC_OK
+
+
 def test_resident_reports_divergence_and_a_missing_cta():
     rng = np.random.default_rng(4)
     M = rng.uniform(-1, 1, (40, 40))
