@@ -960,16 +960,23 @@ static bool fits_l2(int64_t entries, bool mixed) { return (mixed ? 8.0 : 12.0) *
 //     the gathers' latency and costs a longer grid barrier.  FP64: 64^3 10.7 /
 //     11.8, 128^3 37.3 / 37.3, 160^3 70.2 / 66.1; a mixed cycle's FP32 sweeps
 //     (bound by that latency) from about 100,000 rows on: 48^3 4.03 / 3.98, 96^3
-//     13.0 / 10.6, 128^3 25.9 / 21.3, 160^3 48.2 / 38.9;
+//     13.0 / 10.6, 128^3 25.9 / 21.3, 160^3 48.2 / 38.9; a split interface block
+//     (slot rows wait longer) from about 1,000,000: 80^3 in 4x4x4 16.4 / 17.2, 104^3
+//     27.4 / 26.6, 128^3 42.6 / 41.2;
+//   the same, FP64, 2 CTAs/SM, 4 / 2 stages: while the matrix comes from L2 two are
+//     enough and cost less per tile.  74^3 12.18 / 12.05, 80^3 13.69 / 13.54, 88^3
+//     15.9 / 16.0, 100^3 20.4 / 22.4; split, 72^3 14.98 / 14.78, 80^3 16.38 / 16.11;
 //   several lanes (27-point), 4 / 3 / 2 stages: a 26 KB stage holds 78 of the 128
 //     rows of a two-lane tile, a 54 KB one all.  FP64: 32^3 9.6 / 9.5 / 8.6, 64^3
 //     24.5 / 24.3 / 20.7, 128^3 152 / 139 / 127; mixed 48^3 7.1 / 6.6 / 5.8, 64^3
 //     13.6 / 11.7 / 11.5, 96^3 40.7 / 34.7 / 39.0 (FP32 entries take two thirds
 //     of the space, and 36 KB hold the tile).
-static void default_geometry(int lanes, bool mixed, int64_t rows, int* per_sm, int* stages)
+static void default_geometry(int lanes, bool mixed, bool split, int64_t rows, int* per_sm, int* stages)
 {
-    if (lanes == 1) *per_sm = rows >= (mixed ? 100000 : 3000000) ? 3 : 2;
-    else *stages = mixed && rows > 350000 ? 3 : 2;
+    if (lanes == 1) {
+        *per_sm = rows >= (mixed ? 100000 : split ? 1000000 : 3000000) ? 3 : 2;
+        if (!mixed && rows < 600000) *stages = 2;
+    } else *stages = mixed && rows > 350000 ? 3 : 2;
 }
 
 // Row ranges of the resident kernel's CTAs and the dynamic shared memory of the
@@ -1066,7 +1073,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     int stages = o.stages;
     if (c->variant == 2 && c->rows_per_tile == 256 && !o.ctas_per_sm && !o.stages && o.sync == JAC_SYNC_GRID &&
         o.stop == JAC_STOP_GLOBAL)
-        default_geometry(c->lanes, o.precision == JAC_MIXED, rows, &target_per_sm, &stages);
+        default_geometry(c->lanes, o.precision == JAC_MIXED, sp != nullptr, rows, &target_per_sm, &stages);
     if (target_per_sm == 3) c->stages = 3;
     // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
     if (c->variant == 2 && c->rows_per_tile == 256 && target_per_sm == 2 && (stages == 2 || stages == 3))
