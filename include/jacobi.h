@@ -137,7 +137,7 @@ typedef struct {
                                   NULL = row r sits at node r */
     int32_t nrhs;              /* right-hand sides sharing A (1..8, default 1) */
     int32_t transpose;         /* 1 = solve with A^T instead of A (adjoint solves) */
-    int32_t variant;           /* 0 = auto: 2, or, in FP64 with the grid barrier, the global stop, 1 or 2 lanes
+    int32_t variant;           /* 0 = auto: 2, or, in FP64 with the grid barrier, 1 or 2 lanes
                                   per row and no other geometry option, where the matrix fits the
                                   SMs' shared memory, a kernel that keeps it there (jac_stats:
                                   variant 2, ctas_per_sm 1, stages 0); 1 = one launch per sweep (row kernel);
