@@ -940,7 +940,8 @@ inline int64_t nnz_off_of(const ScaledForm& tf) { return tf.rowptr.empty() ? 0 :
 // rounds of gathers and not by its entries (96^3 FP64 57.6 -> 54.1 us a sweep, 61^3
 // mixed 10.0 -> 9.2: the first and last CTAs had a third more rows).  Rows of a
 // substructuring's interface gather from several subdomains: their CTAs took
-// 17 % longer in mixed cycles (131x128x125 in 4x4x4: 22.9 -> 21.6 us).
+// 17 % longer in mixed cycles (131x128x125 in 4x4x4: 22.9 -> 21.6 us; 48x32x55 and
+// 100x90x95 are 1 % slower with it: from 1,500,000 rows on).
 static double form_row_cost(int64_t len, int lanes, bool mixed, bool interface_row)
 {
     if (lanes > 1) return (mixed ? 50.0 : 19.0) + (double)len;
@@ -960,7 +961,9 @@ static bool fits_l2(int64_t entries, bool mixed) { return (mixed ? 8.0 : 12.0) *
 //     the gathers' latency and costs a longer grid barrier.  FP64: 64^3 10.7 /
 //     11.8, 128^3 37.3 / 37.3, 160^3 70.2 / 66.1; a mixed cycle's FP32 sweeps
 //     (bound by that latency) from about 100,000 rows on: 48^3 4.03 / 3.98, 96^3
-//     13.0 / 10.6, 128^3 25.9 / 21.3, 160^3 48.2 / 38.9; a split interface block
+//     13.0 / 10.6, 128^3 25.9 / 21.3, 160^3 48.2 / 38.9 with cycles of 128 sweeps; its
+//     longer barriers and launches count per cycle, so shorter cycles need more rows
+//     (of 32: 118x42x22 7.6 / 8.8, 64^3 10.3 / 11.3); a split interface block
 //     (slot rows wait longer) from about 1,000,000: 80^3 in 4x4x4 16.4 / 17.2, 104^3
 //     27.4 / 26.6, 128^3 42.6 / 41.2;
 //   the same, FP64, 2 CTAs/SM, 4 / 2 stages: while the matrix comes from L2 two are
@@ -971,10 +974,10 @@ static bool fits_l2(int64_t entries, bool mixed) { return (mixed ? 8.0 : 12.0) *
 //     24.5 / 24.3 / 20.7, 128^3 152 / 139 / 127; mixed 48^3 7.1 / 6.6 / 5.8, 64^3
 //     13.6 / 11.7 / 11.5, 96^3 40.7 / 34.7 / 39.0 (FP32 entries take two thirds
 //     of the space, and 36 KB hold the tile).
-static void default_geometry(int lanes, bool mixed, bool split, int64_t rows, int* per_sm, int* stages)
+static void default_geometry(int lanes, bool mixed, int inner, bool split, int64_t rows, int* per_sm, int* stages)
 {
     if (lanes == 1) {
-        *per_sm = rows >= (mixed ? 100000 : split ? 1000000 : 3000000) ? 3 : 2;
+        *per_sm = rows >= (mixed ? 12800000 / std::max(1, inner) : split ? 1000000 : 3000000) ? 3 : 2;
         if (!mixed && rows < 600000) *stages = 2;
     } else *stages = mixed && rows > 350000 ? 3 : 2;
 }
@@ -1073,7 +1076,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     int stages = o.stages;
     if (c->variant == 2 && c->rows_per_tile == 256 && !o.ctas_per_sm && !o.stages && o.sync == JAC_SYNC_GRID &&
         o.stop == JAC_STOP_GLOBAL)
-        default_geometry(c->lanes, o.precision == JAC_MIXED, sp != nullptr, rows, &target_per_sm, &stages);
+        default_geometry(c->lanes, o.precision == JAC_MIXED, o.inner_sweeps, sp != nullptr, rows, &target_per_sm, &stages);
     if (target_per_sm == 3) c->stages = 3;
     // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
     if (c->variant == 2 && c->rows_per_tile == 256 && target_per_sm == 2 && (stages == 2 || stages == 3))
@@ -1232,7 +1235,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     const bool by_form = all_auto && o.sync == JAC_SYNC_GRID && o.stop == JAC_STOP_GLOBAL;
     if (!row_cost && !c->resident && c->variant == 2 && (sp || by_form)) {
         est_cost.resize(rows);
-        const int64_t ifc = plan.splitting == JAC_SUBSTRUCT && !sp ? plan.part_ptr[plan.nparts() - 1] : rows;
+        const int64_t ifc = plan.splitting == JAC_SUBSTRUCT && !sp && rows >= 1500000 ? plan.part_ptr[plan.nparts() - 1] : rows;
         for (int64_t r = 0; r < rows; ++r) {
             const int64_t len = tf.rowptr[r + 1] - tf.rowptr[r];
             est_cost[r] = sp && r >= sp->n_own
