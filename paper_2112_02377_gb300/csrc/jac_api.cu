@@ -940,8 +940,8 @@ inline int64_t nnz_off_of(const ScaledForm& tf) { return tf.rowptr.empty() ? 0 :
 // rounds of gathers and not by its entries (96^3 FP64 57.6 -> 54.1 us a sweep, 61^3
 // mixed 10.0 -> 9.2: the first and last CTAs had a third more rows).  Rows of a
 // substructuring's interface gather from several subdomains: their CTAs took
-// 17 % longer in mixed cycles (131x128x125 in 4x4x4: 22.9 -> 21.6 us; 48x32x55 and
-// 100x90x95 are 1 % slower with it: from 1,500,000 rows on).
+// 17 % longer in mixed cycles (131x128x125 in 4x4x4: 22.9 -> 21.6 us); smaller systems
+// gain nothing from it (FP64 sweeps of 100x90x95 1 % slower): from 1,500,000 rows on.
 static double form_row_cost(int64_t len, int lanes, bool mixed, bool interface_row)
 {
     if (lanes > 1) return (mixed ? 50.0 : 19.0) + (double)len;
@@ -963,7 +963,8 @@ static bool fits_l2(int64_t entries, bool mixed) { return (mixed ? 8.0 : 12.0) *
 //     (bound by that latency) from about 100,000 rows on: 48^3 4.03 / 3.98, 96^3
 //     13.0 / 10.6, 128^3 25.9 / 21.3, 160^3 48.2 / 38.9 with cycles of 128 sweeps; its
 //     longer barriers and launches count per cycle, so shorter cycles need more rows
-//     (of 32: 118x42x22 7.6 / 8.8, 64^3 10.3 / 11.3); a split interface block
+//     (118x42x22 in boxes, of 32 5.01 / 5.32, of 64 4.19 / 4.40; 64^3, of 32 6.79 /
+//     6.79, of 64 5.95 / 5.81; 100x90x95, of 32 13.2 / 11.9); a split interface block
 //     (slot rows wait longer) from about 1,000,000: 80^3 in 4x4x4 16.4 / 17.2, 104^3
 //     27.4 / 26.6, 128^3 42.6 / 41.2;
 //   the same, FP64, 2 CTAs/SM, 4 / 2 stages: while the matrix comes from L2 two are
