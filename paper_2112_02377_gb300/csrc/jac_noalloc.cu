@@ -31,6 +31,7 @@
 #include <string>
 
 #include "../../include/jacobi.h"
+#include "jac_rounds.h"
 
 // cuCtxGetCurrent / cuCtxGetId, fetched through the runtime's driver entry
 // points so that the library does not link libcuda directly.
@@ -170,16 +171,17 @@ __global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* _
     const double bi = i < n ? b[i] : 0.0;
     double s = 0.0, d = 0.0, xi = 0.0;
     bool waited = false;
-    for (int c0 = p0; c0 < p1 || !waited; c0 += kCap) {
-        const int c1 = p1 - c0 < kCap ? p1 : c0 + kCap;
+    jac::for_each_round<kCap>(p0, p1, [&](int first, int count) {
         if (waited) __syncthreads();        // the round before has been read
 #pragma unroll
         for (int q = 0; q < kCap; q += kBlock) {
-            const int at = q + threadIdx.x, e = c0 + at;
-            if (e < c1) {
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(shared_addr(s_val + at)), "l"(val + e)
+            const int at = q + threadIdx.x;
+            if (at < count) {
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(shared_addr(s_val + at)),
+                             "l"(val + first + at)
                              : "memory");
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(shared_addr(s_col + at)), "l"(col + e)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(shared_addr(s_col + at)),
+                             "l"(col + first + at)
                              : "memory");
             }
         }
@@ -188,8 +190,8 @@ __global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* _
         waited = true;
         __syncthreads();
         // this thread's part of the round; the loop ends at the warp's longest
-        const int lo = kb > c0 ? kb : c0, hi = ke < c1 ? ke : c1;
-        const int len = hi > lo ? hi - lo : 0;
+        int from;
+        const int len = jac::row_part(kb, ke, first, count, from);
         const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
         for (int o = 0; o < most; o += kGather) {
             double xv[kGather];
@@ -198,7 +200,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* _
             for (int u = 0; u < kGather; ++u) {
                 j[u] = i;
                 if (o + u < len) {
-                    j[u] = s_col[lo - c0 + o + u];
+                    j[u] = s_col[from + o + u];
                     xv[u] = x[j[u]];
                 }
             }
@@ -206,14 +208,14 @@ __global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* _
             for (int u = 0; u < kGather; ++u) {
                 if (o + u >= most) break;
                 if (o + u < len && j[u] == i) {
-                    d = s_val[lo - c0 + o + u];
+                    d = s_val[from + o + u];
                     xi = xv[u];
                 }
                 // a warp whose rows all have their diagonal here skips the FMA
-                if (__any_sync(0xffffffffu, j[u] != i) && j[u] != i) s = __fma_rn(s_val[lo - c0 + o + u], xv[u], s);
+                if (__any_sync(0xffffffffu, j[u] != i) && j[u] != i) s = __fma_rn(s_val[from + o + u], xv[u], s);
             }
         }
-    }
+    });
     const double t = bi - s;
     if (i < n) y[i] = quotient(t, d);
     if constexpr (LAST) {
