@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
     __shared__ unsigned long long s_mx[2][MW * 32];
     __shared__ ResidentDecision s_dec;
     __shared__ int s_start, s_skip, s_xb, s_words, s_stop, s_done;
-    __shared__ volatile int s_fail;
+    __shared__ volatile int s_fail;          // written by thread 0 between the two CTA barriers of a sweep only
     __shared__ long long s_budget;
     __shared__ double* s_x[NBUF];            // (indexed in shared memory: a local copy would be re-read from L2)
     constexpr int RPS = 32 / L;
@@ -385,7 +385,11 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
         }
         return;
     }
-    // The word that decides sweep j, or the final one (by one lane); false on a timeout.
+    // The word that decides sweep j, or the final one (by one lane); false on a
+    // timeout.  It runs beside the math warps, which may still be reading s_fail, so
+    // it leaves that flag alone: a CTA that got no decision goes on, each later wait
+    // ends at once on ST_TIMEOUT, and thread 0 ends the CTA's loop, between the two
+    // CTA barriers, in the first grid barrier that does not fill.
     auto await_decision = [&](int j, unsigned long long& word) -> bool {
         const long long t0 = clock64();
         int spins = 0;
@@ -393,8 +397,8 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
             word = ld_acquire_u64(&ctl->dec_ready);
             if ((long long)(word & 0xffffffffull) > j || (word >> 32)) return true;
             if ((++spins & 63) == 0) {
-                if (ld_volatile_i32(&ctl->status) & ST_TIMEOUT) { s_fail = 1; return false; }
-                if (clock64() - t0 > budget) { atomicOr(&ctl->status, ST_TIMEOUT); s_fail = 1; return false; }
+                if (ld_volatile_i32(&ctl->status) & ST_TIMEOUT) return false;
+                if (clock64() - t0 > budget) { atomicOr(&ctl->status, ST_TIMEOUT); return false; }
             }
         }
     };
