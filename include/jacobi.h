@@ -17,8 +17,9 @@
  *     (jac_last_error(NULL): the last failure of jac_setup* on this thread).
  *   - Pointers tagged JAC_MEM_HOST are ordinary host memory; JAC_MEM_DEVICE
  *     pointers are device memory on the context's device.  The library
- *     never keeps a caller pointer after the call returns: inputs are
- *     copied, outputs are written before return.
+ *     never keeps a caller pointer after the call returns: inputs have been
+ *     read (vectors of the context's device in place, others through a
+ *     copy) and outputs written before return.
  *   - All device work is issued on the stream given in jac_opts.stream
  *     (NULL = the legacy default stream) and every call that returns results
  *     synchronises that stream before returning.

@@ -252,10 +252,6 @@ cudaError_t allow_smem(const void* fn, int bytes)
     return e;
 }
 
-// A caller's vector of doubles as the kernels read it: device memory in place
-// (nothing is kept after the call), host memory through `stage`.
-jac_status on_device(jac_ctx* c, const double* src, int memory, size_t count, double* stage, const double** out);
-
 jac_status copy_to_stage(jac_ctx* c, const double* src, int memory, size_t count, double* stage)
 {
     if (memory == JAC_MEM_DEVICE) {
@@ -268,13 +264,25 @@ jac_status copy_to_stage(jac_ctx* c, const double* src, int memory, size_t count
     return JAC_OK;
 }
 
-// Device memory that kernels may use in place of a staged copy.
-bool in_place(const double* p, int memory) { return memory == JAC_MEM_DEVICE && ((uintptr_t)p & 7u) == 0; }
+// Device memory that kernels may use in place of a staged copy: the driver is
+// asked who owns it (half a microsecond).
+bool in_place(const jac_ctx* c, const double* p, int memory)
+{
+    if (memory != JAC_MEM_DEVICE) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return usable_in_place(a.type == cudaMemoryTypeDevice, a.device, c->device, (uintptr_t)p);
+}
 
+// A caller's vector of doubles as the kernels read it: in place where that is
+// possible (nothing is kept after the call), else through `stage`.
 jac_status on_device(jac_ctx* c, const double* src, int memory, size_t count, double* stage, const double** out)
 {
     *out = src;
-    if (!src || in_place(src, memory)) return JAC_OK;
+    if (!src || in_place(c, src, memory)) return JAC_OK;
     *out = stage;
     return copy_to_stage(c, src, memory, count, stage);
 }
@@ -2313,7 +2321,7 @@ try {
         CK(c, launch_batched_gather_x(c->d_x[0], c->d_x[1], c->d_row_sys, c->d_mask, c->d_kpar, xb, c->n, c->nrhs,
                                       c->d_d, src, s));
     } else {
-        if (in_place(x, memory)) src = x;
+        if (in_place(c, x, memory)) src = x;
         CK(c, launch_scatter_rows(c->d_perm, c->d_x[xb], c->d_d, src, (int)c->n, s));
     }
     if (src == x) {
@@ -2377,7 +2385,7 @@ try {
     // (dA over lambda or x goes through the staged copies)
     const uintptr_t g0 = (uintptr_t)dA, g1 = g0 + (size_t)c->nnz * 8;
     auto apart = [&](const double* p) { return (uintptr_t)p + (size_t)c->n * 8 <= g0 || g1 <= (uintptr_t)p; };
-    const bool direct = in_place(lambda, memory) && in_place(x, memory) && in_place(dA, memory) && apart(lambda) &&
+    const bool direct = in_place(c, lambda, memory) && in_place(c, x, memory) && in_place(c, dA, memory) && apart(lambda) &&
                         apart(x);
     if (!direct && !c->d_stage2) CK(c, dalloc(&c->d_stage2, c->n + 16));
     if (!direct && !c->d_grad) CK(c, dalloc(&c->d_grad, (size_t)c->nnz + 16));

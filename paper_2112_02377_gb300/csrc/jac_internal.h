@@ -9,6 +9,15 @@
 
 namespace jac {
 
+// Whether kernels on `device` may dereference a caller's device vector: only
+// memory of that device (another GPU's may not be mapped there, managed or host
+// memory may have to be migrated or be unreachable) at a double's alignment.
+// Everything else is copied, which takes whatever cudaMemcpy takes.
+inline bool usable_in_place(bool device_memory, int owner, int device, uintptr_t p)
+{
+    return device_memory && owner == device && (p & 7u) == 0;
+}
+
 // A square matrix in 0-based CSR, host memory.
 struct HostCSR {
     int64_t n = 0;
