@@ -106,28 +106,54 @@ __device__ __forceinline__ unsigned shared_addr(const void* p)
     return (unsigned)__cvta_generic_to_shared(p);
 }
 
-// t / d in five FP64 operations where IEEE division takes about twice as many,
-// on a chip whose FP64 pipe bounds the sweep: a single-precision reciprocal of d
-// (its leading bits, moved between the formats with integer operations), one
-// Newton step, and Markstein's quotient correction (Markstein, IBM J. Res. Dev.
-// 34 (1990) 111): q = t r, q + (t - d q) r.  r is good to 2^-44, so the value
-// rounded in the last operation is within 2^-86 of t / d.  Outside exponents
-// that keep every step normal, and for t = 0, the division itself.
+// t / d, correctly rounded, in five FP64 operations where the division takes about
+// twice as many, on a chip whose FP64 pipe bounds the sweep: a single-precision
+// reciprocal of d (its leading bits, moved between the formats with integer
+// operations), one Newton step, and Markstein's quotient correction (Markstein, IBM
+// J. Res. Dev. 34 (1990) 111): q = t r, z = q + (t - d q) r.  r is good to 2^-44 and
+// the value rounded to z within 2^-33 of an ulp of t / d, so z is right unless that
+// value lies as close to a midpoint.  Two tests find that out:
+//   in single precision, beside the FP64 pipe: the correction c = (t - d q) r in ulps
+//     of q, at most 2^9 and good to 2^-12, against the ulps that the rounding moved;
+//   for the one quotient in 2,000 next to a midpoint (or past the end of q's
+//     binade): t - d z, exact in one FMA for z within an ulp of t / d, is below half
+//     an ulp of z times |d| exactly where z is the nearest number.
+// Where neither passes, where z is a power of two (its lower neighbour is nearer),
+// outside exponents that keep every step normal, and for t = 0, the division itself.
+// 3,374,850 rows, us a sweep: without the tests 92.2, both 93.3, the exact one for
+// every row 96.0, the first alone 96.2 (a warp in 60 divides), IEEE division 105.
 __device__ __forceinline__ double quotient(double t, double d)
 {
     const unsigned dh = (unsigned)__double2hiint(d), dl = (unsigned)__double2loint(d);
     const unsigned th = (unsigned)__double2hiint(t);
     const unsigned de = (dh >> 20) & 0x7ffu, te = (th >> 20) & 0x7ffu;
-    if (de - 923u > 200u || te - 200u > 1600u) return t / d;     // |d| in 2^-100 .. 2^100, |t| in 2^-823 .. 2^777
-    const float f = __uint_as_float((dh & 0x80000000u) | (((dh & 0x7fffffffu) - (896u << 20)) << 3) | (dl >> 29));
-    float rf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
-    const unsigned rb = __float_as_uint(rf);
-    const double r0 = __hiloint2double((int)((rb & 0x80000000u) | (((rb & 0x7fffffffu) >> 3) + (896u << 20))),
-                                       (int)(rb << 29));
-    const double r = __fma_rn(__fma_rn(-d, r0, 1.0), r0, r0);
-    const double q = __dmul_rn(t, r);
-    return __fma_rn(__fma_rn(-d, q, t), r, q);
+    if (de - 923u <= 200u && te - 200u <= 1600u) {               // |d| in 2^-100 .. 2^101, |t| in 2^-823 .. 2^778
+        const float f = __uint_as_float((dh & 0x80000000u) | (((dh & 0x7fffffffu) - (896u << 20)) << 3) | (dl >> 29));
+        float rf;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+        const unsigned rb = __float_as_uint(rf);
+        const double r0 = __hiloint2double((int)((rb & 0x80000000u) | (((rb & 0x7fffffffu) >> 3) + (896u << 20))),
+                                           (int)(rb << 29));
+        const double r = __fma_rn(__fma_rn(-d, r0, 1.0), r0, r0);
+        const double q = __dmul_rn(t, r);
+        const double rem = __fma_rn(-d, q, t);
+        const double z = __fma_rn(rem, r, q);
+        // rem r in ulps of q, in single precision, and the ulps that the rounding took
+        const unsigned mh = (unsigned)__double2hiint(rem), qh = (unsigned)__double2hiint(q);
+        const unsigned zh = (unsigned)__double2hiint(z), zl = (unsigned)__double2loint(z);
+        const unsigned me = (mh >> 20) & 0x7ffu, qe = (qh >> 20) & 0x7ffu;
+        const unsigned mb = __funnelshift_l((unsigned)__double2loint(rem), mh & 0x7fffffffu, 3) - ((te - 179u) << 23);
+        const float m = me + 179u > te ? __uint_as_float(mb | ((mh ^ th) & 0x80000000u)) : 0.0f;
+        const float c = __fmul_rn(m, __uint_as_float((rb & 0x7fffffffu) + ((te - qe) << 23)));
+        const float off = __fsub_rn(c, (float)(int)(zl - (unsigned)__double2loint(q)));
+        const bool plain = ((zh ^ qh) & 0xfff00000u) == 0 && ((zh & 0xfffffu) | zl) != 0;
+        if (plain && fabsf(off) < 0.4997f) return z;
+        const int back = __double2hiint(__fma_rn(-d, z, t)) & 0x7fffffff;
+        // high word of |d| 2^(e - 53), e the exponent of z (at least 2^-1001)
+        const int half = (int)((dh & 0x7fffffffu) + (zh & 0x7ff00000u) - (1076u << 20));
+        if (back < half && ((zh & 0xfffffu) | zl)) return z;
+    }
+    return t / d;
 }
 
 // One sweep on a CSR matrix that stores its diagonal, one thread per row:
@@ -150,9 +176,9 @@ __device__ __forceinline__ double quotient(double t, double d)
 //
 // Bound by the FP64 pipe (six FMAs, a subtraction and the quotient's five
 // operations per 7-point row) with the 104 bytes a row moves close behind: about
-// 60 us each for 3,374,850 rows, which take 91 us a sweep (105 with IEEE
-// division; 3,050 before rows were staged); 110,544 rows 7.2 us, 1,188 rows
-// 3.3 us.  Five blocks an SM (48 registers) measured best, seven gathers
+// 60 us each for 3,374,850 rows, which take 93 us a sweep (105 with IEEE
+// division; 3,050 before rows were staged); 110,592 rows 8.2 us, 1,188 rows
+// 4.0 us.  Five blocks an SM (48 registers) measured best, seven gathers
 // together as good as eight; a block that copies its next tile while it sums one
 // (two buffers, four blocks) took 105 us.
 template <bool LAST>
