@@ -141,7 +141,9 @@ typedef struct {
     int32_t variant;           /* 0 = auto: 2, or, in FP64 with the grid barrier, 1 or 2 lanes
                                   per row and no other geometry option, where the matrix fits the
                                   SMs' shared memory, a kernel that keeps it there (jac_stats:
-                                  variant 2, ctas_per_sm 1, stages 0); 1 = one launch per sweep (row kernel);
+                                  variant 2, ctas_per_sm 1, stages 0; calls of one or two sweeps, which a
+                                  launch of it costs more than it gains, run as variant 2 where
+                                  the matrix is large); 1 = one launch per sweep (row kernel);
                                   2 = persistent grid-synchronised pipelined kernel, x gathered
                                   through L1/L2; 3 = as 2 with each tile's x halo (its dependency list,
                                   Sec. 4.2.2) staged into shared memory */
@@ -385,7 +387,8 @@ jac_status jac_adjoint_grad(jac_ctx* ctx, const double* lambda, const double* x,
  * tiles, wait_ms[i] = time it spent in the grid barrier, summed over sweeps.
  * The GPU counterpart of the paper's communication / total time columns
  * (Sec. 5.2 tables).  Host arrays of `max` entries (may be NULL);
- * *ctas receives the CTA count (0 for the one-launch-per-sweep variant).
+ * *ctas receives the CTA count of that call (0 for the one-launch-per-sweep
+ * variant).
  */
 jac_status jac_get_trace(jac_ctx* ctx, double* compute_ms, double* wait_ms, int64_t max, int64_t* ctas);
 

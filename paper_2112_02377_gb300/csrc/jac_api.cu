@@ -30,6 +30,15 @@ namespace jac {
 void record_thread_error(const std::string& msg) { g_setup_error = msg; }
 }  // namespace jac
 
+// A second geometry for FP64 sweeps (pipelined kernel, 256 threads, grid barrier): the
+// calls for which the context's own is the slower one (second_geometry).
+struct SecondGeometry {
+    const void* fn = nullptr;      // nullptr: none
+    int64_t most = 0;              // sweeps of the longest call that runs in it
+    int grid = 0, threads = 0, smem = 0, ntiles = 0, emax = 0;
+    int *d_row0 = nullptr, *d_nnz0 = nullptr, *d_cta0 = nullptr;
+};
+
 struct jac_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -57,6 +66,8 @@ struct jac_ctx {
     bool keep_l2 = false;          // the matrix stays in L2 from sweep to sweep
     bool resident = false;         // FP64 sweeps run in the resident kernel
     int* d_cta_row = nullptr;      // resident kernel: ctas+1 first rows
+    SecondGeometry second;
+    int trace_ctas = 0;            // CTAs of the last call's geometry
     bool ns = false;               // neighbour-synchronised FP64 sweeps
     int sync = JAC_SYNC_GRID;      // jac_sync of the FP64 kernel
     bool certify = false;          // asynchronous contexts: run the grid-synchronised kernel
@@ -361,6 +372,21 @@ DevTiles devtiles(const jac_ctx* c)
     return t;
 }
 
+DevTiles second_tiles(const jac_ctx* c)
+{
+    const SecondGeometry& g = c->second;
+    DevTiles t{};
+    t.row0 = g.d_row0;
+    t.nnz0 = g.d_nnz0;
+    t.row1 = g.d_row0 + 1;
+    t.nnz1 = g.d_nnz0 + 1;
+    t.cta0 = g.d_cta0;
+    t.ntiles = g.ntiles;
+    t.keep = c->keep_l2 ? 1 : 0;
+    t.emax = g.emax;
+    return t;
+}
+
 DevBatch devbatch(const jac_ctx* c)
 {
     DevBatch b;
@@ -392,7 +418,7 @@ int mixed_cycles_per_step(const jac_ctx* c)
 }
 
 // FP64 sweeps of a graph step.  The resident kernel loads the matrix and ends
-// with a barrier of its own in every launch (about 10 us together), against 2 us
+// with a barrier of its own in every launch (3 to 9 us together), against 2 us
 // a sweep: its steps have at least 512 sweeps.
 int sweeps_per_step(const jac_ctx* c) { return c->resident ? std::max(c->K, 512) : c->K; }
 
@@ -455,6 +481,22 @@ jac_status enqueue_step(jac_ctx* c, bool mixed)
             for (int j = 1; j < m - 1; ++j) CK(c, launch_row_sweep(PH_P32, devmat(c), devvec(c), c->d_ctl, s));
             CK(c, launch_row_sweep(PH_P32L, devmat(c), devvec(c), c->d_ctl, s));
         }
+    }
+    return JAC_OK;
+}
+
+// Whether a call of at most `sweeps` FP64 sweeps runs in the second geometry.
+bool use_second(const jac_ctx* c, int64_t sweeps) { return c->second.fn && sweeps <= c->second.most; }
+
+// `sweeps` FP64 sweeps in the second geometry.
+jac_status second_step(jac_ctx* c, int64_t sweeps)
+{
+    cudaStream_t s = stream_of(c);
+    const SecondGeometry& g = c->second;
+    for (int64_t left = sweeps; left > 0; left -= c->K) {
+        CK(c, launch_reset_bar(c->d_ctl, s));
+        CK(c, launch_persistent(g.fn, g.grid, g.threads, g.smem, devmat(c), devvec(c), second_tiles(c), c->d_ctl,
+                                (int)std::min<int64_t>(left, c->K), s));
     }
     return JAC_OK;
 }
@@ -579,7 +621,7 @@ jac_status status_from_ctl(jac_ctx* c, const JacCtl& h)
 jac_status arm(jac_ctx* c, int test, int mixed, long long k_limit, long long k_delta, double tol)
 {
     if (c->d_trace)
-        CK(c, cudaMemsetAsync(c->d_trace, 0, 4 * sizeof(unsigned long long) * c->grid, stream_of(c)));
+        CK(c, cudaMemsetAsync(c->d_trace, 0, 4 * sizeof(unsigned long long) * c->nslots, stream_of(c)));
     if (c->d_loc)
         CK(c, cudaMemsetAsync(c->d_loc, 0, loc_slots(c) * sizeof(unsigned long long) * c->nloc, stream_of(c)));
     CK(c, launch_arm(c->d_ctl, test, mixed, c->o.inner_sweeps, k_limit, k_delta, tol, c->o.norm, c->d_hist, c->hist_cap,
@@ -607,6 +649,7 @@ void destroy(jac_ctx* c)
     dfree(c->d_rowptr); dfree(c->d_col); dfree(c->d_S64); dfree(c->d_S32); dfree(c->d_b); dfree(c->d_d);
     dfree(c->d_x[0]); dfree(c->d_x[1]); dfree(c->d_x[2]); dfree(c->d_x[3]); dfree(c->d_x[4]);
     dfree(c->d_cta_row);
+    dfree(c->second.d_row0); dfree(c->second.d_nnz0); dfree(c->second.d_cta0);
     dfree(c->d_dep_ptr); dfree(c->d_dep); dfree(c->d_done); dfree(c->d_e[0]); dfree(c->d_e[1]); dfree(c->d_dlt);
     dfree(c->d_part); dfree(c->d_ctl); dfree(c->d_hist); dfree(c->d_perm); dfree(c->d_stage); dfree(c->d_stage2);
     dfree(c->d_bmap); dfree(c->d_slot_info);
@@ -1017,6 +1060,68 @@ static int64_t resident_plan(const ScaledForm& tf, const Plan& plan, int ctas, i
     return most;
 }
 
+// Entries that a pipeline stage holds for a tile of `rows` rows: variant 2 has 2
+// CTAs/SM x 4 stages for 224/256-thread tiles (or 3 / 2 larger stages), 3 CTAs/SM x 3
+// stages, 1 CTA/SM x 4 stages for 480-row tiles.
+static int stage_entries(int tile_rows, int rows, int per_sm, int stages, int64_t max_off)
+{
+    int64_t budget = tile_rows <= 256 ? 26 * 1024 : 52 * 1024;
+    if (tile_rows == 256 && per_sm == 2 && stages == 3) budget = 36 * 1024;
+    if (tile_rows == 256 && per_sm == 2 && stages == 2) budget = 54 * 1024;
+    const int64_t fit = std::max<int64_t>(rows, (budget - 16 * rows - 1024) / 12);
+    return (int)std::min<int64_t>(std::max<int64_t>(1, max_off) * rows, fit);
+}
+
+// Sets up the second geometry of a context (per_sm CTAs/SM, stages) for calls of at
+// most `most` FP64 sweeps; where it cannot be had every call keeps the first.
+static jac_status second_geometry(jac_ctx* c, const Plan& plan, const ScaledForm& tf, int per_sm, int stages, int64_t most,
+                                  const std::vector<double>* row_cost, int sms)
+{
+    const int rows = 256 / c->lanes;
+    SecondGeometry g;
+    g.most = most;
+    g.threads = persistent_threads(256);
+    g.emax = stage_entries(256, rows, per_sm, stages, tf.max_off);
+    g.smem = persistent_smem_bytes(rows, g.emax, stages);
+    const void* fn = persistent_kernel(256, stages, false, c->lanes, c->stop == JAC_STOP_LOCAL ? 4 : JAC_SYNC_GRID);
+    int fits = 0;
+    if (!fn || allow_smem(fn, g.smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, fn, g.threads, g.smem) != cudaSuccess || fits < 1) {
+        cudaGetLastError();
+        return JAC_OK;
+    }
+    g.grid = std::min(fits, per_sm) * sms;
+    Tiling t;
+    make_tiling(tf, plan, rows, g.emax, g.grid, t, row_cost);
+    g.ntiles = (int)t.ntiles();
+    auto upload = [&](int** d, const std::vector<int32_t>& v) -> jac_status {
+        CK(nullptr, dalloc(d, v.size()));
+        CK(nullptr, cudaMemcpy(*d, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        return JAC_OK;
+    };
+    jac_status st = upload(&c->second.d_row0, t.row0);
+    if (st == JAC_OK) st = upload(&c->second.d_nnz0, t.nnz0);
+    if (st == JAC_OK) st = upload(&c->second.d_cta0, t.cta0);
+    if (st != JAC_OK) return st;
+    g.d_row0 = c->second.d_row0;
+    g.d_nnz0 = c->second.d_nnz0;
+    g.d_cta0 = c->second.d_cta0;
+    g.fn = fn;
+    c->second = g;
+    return JAC_OK;
+}
+
+// Sweeps of the longest call that the resident kernel loses to the pipelined one: a
+// launch of it first loads the matrix and ends with a barrier and a decision of its
+// own, some 3 us and 30 ns per KB of a CTA's shared memory, and gains about 4 us a
+// sweep.  jac_sweep of 1 / 2 / 3 sweeps, us on the device (in steps of two), resident
+// / pipelined: 7-point 16^3 16.5 / 16.5, 18.5 / 22.6, 20.6 / 28.8; 48^3 (63 KB)
+// 20.6 / 18.5, 22.7 / 26.7; 64^3 (150 KB) 24.7 / 20.6, 30.8 / 30.8, 37.0 / 41.1; 70^3
+// (196 KB) 28.7 / 22.6, 34.9 / 34.9, 43.1 / 45.2; 27-point 44^3 (180 KB) 30.9 / 22.6,
+// 39.0 / 34.9, 45.2 / 47.2.  jac_solve counts one more than the sweeps that
+// maxit leaves it: a solve that its tolerance ends early cannot be known beforehand.
+static int resident_short_calls(int64_t smem) { return smem > 170 * 1024 ? 2 : smem > 34 * 1024 ? 1 : 0; }
+
 // A context from a matrix already split and scaled: tf holds the kernel rows
 // (tf.n of them; n for jac_setup, more with a split interface block), tf.d and
 // the iterate the n rows.  sp: the split interface layout (jac_setup_local),
@@ -1090,6 +1195,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
     if (c->variant == 2 && c->rows_per_tile == 256 && target_per_sm == 2 && (stages == 2 || stages == 3))
         c->stages = stages;
+    const int pipelined_stages = c->stages;
     // ---- the resident kernel, where the caller leaves the geometry open and the matrix fits
     bool all_auto = o.variant == 0 && !o.tile_rows && !o.ctas_per_sm && !o.stages;
     const bool local_stop = o.stop == JAC_STOP_LOCAL;
@@ -1120,23 +1226,17 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     }
     if (c->variant >= 2 && !c->resident) {
         const int rows = c->rows_per_tile / c->lanes;     // rows of a tile
-        int64_t cap_entries = (int64_t)std::max<int64_t>(1, tf.max_off) * rows;
-        int64_t stage_budget;
         if (c->variant == 3) {
             // 2 CTAs/SM x 3 stages of (matrix data + run list + x window) in ~210 KB
             c->stages = 3;
             c->xcap = 1280;
             c->maxruns = 16;
-            stage_budget = 36 * 1024 - (c->xcap + 8) * 8;
+            const int64_t stage_budget = 36 * 1024 - (c->xcap + 8) * 8;
+            c->emax = (int)std::min<int64_t>(std::max<int64_t>(1, tf.max_off) * rows,
+                                             std::max<int64_t>(rows, (stage_budget - 16 * rows - 1024) / 12));
         } else {
-            // 2 CTAs/SM x 4 stages for 224/256-thread tiles (or 3 / 2 larger
-            // stages), 3 CTAs/SM x 3 stages, 1 CTA/SM x 4 stages for 480-row tiles
-            stage_budget = c->rows_per_tile <= 256 ? 26 * 1024 : 52 * 1024;
-            if (c->rows_per_tile == 256 && target_per_sm == 2 && c->stages == 3) stage_budget = 36 * 1024;
-            if (c->rows_per_tile == 256 && target_per_sm == 2 && c->stages == 2) stage_budget = 54 * 1024;
+            c->emax = stage_entries(c->rows_per_tile, rows, target_per_sm, c->stages, tf.max_off);
         }
-        const int64_t budget_entries = std::max<int64_t>(rows, (stage_budget - 16 * rows - 1024) / 12);
-        c->emax = (int)std::min<int64_t>(cap_entries, budget_entries);
         if (c->variant == 3) {
             c->pfn64 = halo_kernel(c->stages, false);
             c->pfnmix = halo_kernel(c->stages, true);
@@ -1300,7 +1400,18 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         }
         c->dep_edges = (int64_t)dep.size();
     }
-    c->nslots = c->grid;
+    // short calls of a resident context: the geometry it would have without
+    const int short_calls = c->resident ? resident_short_calls(c->smem) : 0;
+    if (short_calls > 0) {
+        if (c->lanes > 1 && c->stop == JAC_STOP_GLOBAL) {
+            est_cost.resize(rows);
+            for (int64_t r = 0; r < rows; ++r) est_cost[r] = form_row_cost(tf.rowptr[r + 1] - tf.rowptr[r], c->lanes, false, false);
+        }
+        st = second_geometry(C, plan, tf, target_per_sm, pipelined_stages, short_calls,
+                             est_cost.empty() ? nullptr : &est_cost, prop.multiProcessorCount);
+        if (st != JAC_OK) return st;
+    }
+    c->nslots = std::max(c->grid, c->second.grid);
 
     // ---- device buffers
     CK(nullptr, dalloc(&c->d_rowptr, rows + 1 + 16));
@@ -1355,7 +1466,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
             CK(nullptr, cudaMemcpy(c->d_mem_part, mem_part.data(), mem_part.size() * 4, cudaMemcpyHostToDevice));
         CK(nullptr, cudaMemset(c->d_loc, 0, loc_slots(c.get()) * sizeof(unsigned long long) * c->nloc));
     }
-    if (c->variant >= 2) CK(nullptr, dalloc(&c->d_trace, 4 * (size_t)c->grid));
+    if (c->variant >= 2) CK(nullptr, dalloc(&c->d_trace, 4 * (size_t)c->nslots));
     CK(nullptr, dalloc(&c->d_ctl, 1));
     CK(nullptr, dalloc(&c->d_stage, n + 16));
     CK(nullptr, cudaMallocHost((void**)&c->h_ctl, 2 * sizeof(JacCtl)));
@@ -1447,7 +1558,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     const double* bd = nullptr;
     st = on_device(C, b, b_memory, (size_t)n, c->d_stage, &bd);
     if (st != JAC_OK) return fail(nullptr, st, C->err);
-    CK(nullptr, launch_gather_b(sp ? c->d_bmap : c->d_perm, bd, c->d_b, (int)rows, c->d_part, 2 * c->nslots, c->d_ctl,
+    CK(nullptr, launch_gather_b(sp ? c->d_bmap : c->d_perm, bd, c->d_b, (int)rows, c->d_part, 2 * c->grid, c->d_ctl,
                                 sm));
     CK(nullptr, launch_reset_iterate(c->d_ctl, sm));
     CK(nullptr, launch_arm(c->d_ctl, 0, 0, o.inner_sweeps, 0, 0, -1.0, o.norm, c->d_hist, c->hist_cap, (long long)o.timeout_cycles,
@@ -2103,7 +2214,7 @@ try {
     const double* bd = nullptr;
     const jac_status st = on_device(c, b, memory, (size_t)c->n, c->d_stage, &bd);
     if (st != JAC_OK) return st;
-    CK(c, launch_gather_b(c->split ? c->d_bmap : c->d_perm, bd, c->d_b, (int)c->rows, c->d_part, 2 * c->nslots, c->d_ctl,
+    CK(c, launch_gather_b(c->split ? c->d_bmap : c->d_perm, bd, c->d_b, (int)c->rows, c->d_part, 2 * c->grid, c->d_ctl,
                           s));
     CK(c, s ? cudaStreamSynchronize(s) : cudaDeviceSynchronize());
     return JAC_OK;
@@ -2127,10 +2238,12 @@ try {
     }
     jac_status st = arm(c, 0, 0, 0, k, -1.0);
     if (st != JAC_OK) return st;
-    const int launches = (int)(((int64_t)k + sweeps_per_step(c) - 1) / sweeps_per_step(c));
+    const bool second = use_second(c, k);
+    const int launches = second ? 1 : (int)(((int64_t)k + sweeps_per_step(c) - 1) / sweeps_per_step(c));
+    c->trace_ctas = second ? c->second.grid : c->grid;
     CK(c, cudaEventRecord(c->ev0, s));
     for (int i = 0; i < launches; ++i) {
-        st = run_graph(c, false);
+        st = second ? second_step(c, k) : run_graph(c, false);
         if (st != JAC_OK) return st;
     }
     CK(c, cudaEventRecord(c->ev1, s));
@@ -2188,6 +2301,10 @@ static jac_status solve_impl(jac_ctx* c, double tol, int64_t maxit, int64_t* swe
     }
     jac_status st = arm(c, 1, mixed ? 1 : 0, maxit, -1, tol);
     if (st != JAC_OK) return st;
+    const int64_t rest = std::max<int64_t>(0, maxit - c->h_ctl[0].k);   // it evaluates at most rest + 1 iterates
+    const bool second = !mixed && rest < INT32_MAX && use_second(c, rest + 1);
+    c->trace_ctas = second ? c->second.grid : c->grid;
+    auto step = [&]() { return second ? second_step(c, rest + 1) : run_graph(c, mixed); };
     CK(c, cudaEventRecord(c->ev0, s));
     // Launch graph steps, keeping one step in flight while the previous
     // step's control block is inspected on the host.
@@ -2206,7 +2323,7 @@ static jac_status solve_impl(jac_ctx* c, double tol, int64_t maxit, int64_t* swe
     CK(c, cudaEventCreateWithFlags(&ev.b, cudaEventDisableTiming));
     cudaEvent_t& ea = ev.a;
     cudaEvent_t& eb = ev.b;
-    st = run_graph(c, mixed);
+    st = step();
     if (st == JAC_OK) st = fetch_ctl(c, ha);
     if (st != JAC_OK) return st;
     cudaEventRecord(ea, s);
@@ -2225,7 +2342,7 @@ static jac_status solve_impl(jac_ctx* c, double tol, int64_t maxit, int64_t* swe
             cudaStreamSynchronize(s);
             return fail(c, JAC_ECUDA, "the sweep loop did not terminate within its step bound");
         }
-        st = run_graph(c, mixed);
+        st = step();
         if (st == JAC_OK) st = fetch_ctl(c, hb);
         if (st != JAC_OK) return st;
         cudaEventRecord(eb, s);
@@ -2411,12 +2528,13 @@ try {
 jac_status jac_get_trace(jac_ctx* c, double* compute_ms, double* wait_ms, int64_t max, int64_t* ctas)
 try {
     if (!c || !ctas) return JAC_EINVAL;
-    *ctas = c->d_trace ? c->grid : 0;
+    const int last = c->trace_ctas ? c->trace_ctas : c->grid;
+    *ctas = c->d_trace ? last : 0;
     if (!c->d_trace || max <= 0) return JAC_OK;
     DeviceGuard g(c->device);
-    std::vector<unsigned long long> h(4 * (size_t)c->grid);
+    std::vector<unsigned long long> h(4 * (size_t)last);
     CK(c, cudaMemcpy(h.data(), c->d_trace, h.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost));
-    const int64_t m = std::min<int64_t>(max, c->grid);
+    const int64_t m = std::min<int64_t>(max, last);
     for (int64_t i = 0; i < m; ++i) {
         if (compute_ms) compute_ms[i] = h[4 * i] * 1e-6;
         if (wait_ms) wait_ms[i] = h[4 * i + 1] * 1e-6;

@@ -357,20 +357,34 @@ void make_tiling(const ScaledForm& tf, const Plan& plan, int32_t rows_per_tile, 
     const int64_t n = r_end < 0 ? tf.n : r_end;
     const int64_t b0 = r_begin;
     // CTA row ranges: contiguous, cut at row granularity so that every CTA
-    // carries the same estimated cost (pre[r - b0]: cost of rows b0 .. r-1).
-    std::vector<double> pre(n - b0 + 1, 0.0);
-    for (int64_t r = b0; r < n; ++r) {
-        const double w = row_cost ? (*row_cost)[r] : default_row_cost(tf.rowptr[r + 1] - tf.rowptr[r]);
-        pre[r - b0 + 1] = pre[r - b0] + w;
+    // carries the same estimated cost (pre(r): cost of rows b0 .. r-1; the default
+    // model is affine in the entries, so its sums need no pass over the rows).
+    std::vector<double> acc;
+    if (row_cost) {
+        acc.assign(n - b0 + 1, 0.0);
+        for (int64_t r = b0; r < n; ++r) acc[r - b0 + 1] = acc[r - b0] + (*row_cost)[r];
     }
+    const double row_part = default_row_cost(0);
+    auto pre = [&](int64_t r) -> double {
+        return row_cost ? acc[r - b0] : row_part * (double)(r - b0) + (double)(tf.rowptr[r] - tf.rowptr[b0]);
+    };
     std::vector<int64_t> rb(ctas + 1, b0);
     rb[ctas] = n;
     {
         int64_t cur = b0;
-        const double tot = pre[n - b0];
+        const double tot = pre(n);
         for (int64_t g = 1; g < ctas; ++g) {
             const double target = tot * (double)g / (double)ctas;
-            while (cur < n && pre[cur - b0] + 0.5 * (pre[cur - b0 + 1] - pre[cur - b0]) < target) ++cur;
+            auto before = [&](int64_t r) { return pre(r) + 0.5 * (pre(r + 1) - pre(r)) < target; };
+            if (row_cost) {
+                while (cur < n && before(cur)) ++cur;
+            } else {   // whole numbers and halves: exact, so bisection finds the same row
+                for (int64_t hi = n; cur < hi;) {
+                    const int64_t mid = cur + (hi - cur) / 2;
+                    if (before(mid)) cur = mid + 1;
+                    else hi = mid;
+                }
+            }
             cur = aligned_up(cur);
             rb[g] = cur;
         }
@@ -388,14 +402,13 @@ void make_tiling(const ScaledForm& tf, const Plan& plan, int32_t rows_per_tile, 
         while (r < end) {
             while (p + 1 < P && plan.part_ptr[p + 1] <= r) ++p;
             const int64_t lim = std::min<int64_t>(end, plan.part_ptr[p + 1]);
-            int64_t rows = 0, ent = 0;
-            while (r + rows < lim && rows < rows_per_tile) {
-                const int64_t len = tf.rowptr[r + rows + 1] - tf.rowptr[r + rows];
-                if (rows > 0 && ent + len > max_entries) break;
-                ent += len;
-                ++rows;
-                if (ent > max_entries) break;   // a single oversized row forms its own tile
-            }
+            // as many rows as fit; a single oversized row forms its own tile
+            const int64_t most = std::min<int64_t>(lim - r, rows_per_tile);
+            const int64_t full = (int64_t)tf.rowptr[r] + max_entries;
+            int64_t rows = std::upper_bound(tf.rowptr.begin() + r + 1, tf.rowptr.begin() + r + most + 1, full,
+                                            [](int64_t v, int32_t at) { return v < at; }) -
+                           (tf.rowptr.begin() + r + 1);
+            rows = std::max<int64_t>(rows, 1);
             if (align > 1 && r >= align_from && r + rows < lim && (r + rows - align_from) % align) {
                 // aligned cut: back to the previous boundary, or on to the next one
                 // (the tile then exceeds the staged entries and is read from L2)
