@@ -1188,8 +1188,9 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     }
     int target_per_sm = (c->variant == 2 && c->rows_per_tile == 256 && o.ctas_per_sm == 3) ? 3 : 2;
     int stages = o.stages;
-    if (c->variant == 2 && c->rows_per_tile == 256 && !o.ctas_per_sm && !o.stages && o.sync == JAC_SYNC_GRID &&
-        o.stop == JAC_STOP_GLOBAL)
+    const bool open = c->variant == 2 && c->rows_per_tile == 256 && !o.ctas_per_sm && !o.stages &&
+                      o.sync == JAC_SYNC_GRID && o.stop == JAC_STOP_GLOBAL;
+    if (open)
         default_geometry(c->lanes, o.precision == JAC_MIXED, o.inner_sweeps, sp != nullptr, rows, &target_per_sm, &stages);
     if (target_per_sm == 3) c->stages = 3;
     // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
@@ -1410,6 +1411,18 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         st = second_geometry(C, plan, tf, target_per_sm, pipelined_stages, short_calls,
                              est_cost.empty() ? nullptr : &est_cost, prop.multiProcessorCount);
         if (st != JAC_OK) return st;
+    }
+    // FP64 sweeps of a mixed context (jac_sweep) whose cycles run best with a third
+    // CTA per SM, which those sweeps do not: they take an FP64 context's geometry.
+    // us a sweep in the cycles' / there: 7-point 48^3 8.8 / 7.3, 64^3 11.1 / 9.9, 80^3
+    // 15.0 / 13.6, 128^3 36.7 / 36.6; one sweep alone 100^3 37.0 / 35.5, 128^3 51.4 / 49.8.
+    if (open && o.precision == JAC_MIXED && c->variant == 2 && c->lanes == 1 && target_per_sm == 3) {
+        int per_sm = 2, fp64_stages = 4;
+        default_geometry(c->lanes, false, o.inner_sweeps, false, rows, &per_sm, &fp64_stages);
+        if (per_sm == 2) {
+            st = second_geometry(C, plan, tf, per_sm, fp64_stages, INT32_MAX, nullptr, prop.multiProcessorCount);
+            if (st != JAC_OK) return st;
+        }
     }
     c->nslots = std::max(c->grid, c->second.grid);
 
