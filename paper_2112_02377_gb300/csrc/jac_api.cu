@@ -1006,16 +1006,46 @@ static double form_row_cost(int64_t len, int lanes, bool mixed, bool interface_r
 // 12.9 / 12.2, 112^3 (66 MB) 15.5 / 15.6; 27-point mixed 64^3 (51 MB) 10.7 / 10.3.
 static bool fits_l2(int64_t entries, bool mixed) { return (mixed ? 8.0 : 12.0) * (double)entries <= 64e6; }
 
+// Entries that a pipeline stage holds for a tile of `rows` rows: variant 2 has 2
+// CTAs/SM x 4 stages for 224/256-thread tiles (or 3 / 2 larger stages), 3 CTAs/SM x 3
+// stages, 1 CTA/SM x 4 stages for 480-row tiles.
+static int stage_entries(int tile_rows, int rows, int per_sm, int stages, int64_t max_off)
+{
+    int64_t budget = tile_rows <= 256 ? 26 * 1024 : 52 * 1024;
+    if (tile_rows == 256 && per_sm == 2 && stages == 3) budget = 36 * 1024;
+    if (tile_rows == 256 && per_sm == 2 && stages == 2) budget = 54 * 1024;
+    const int64_t fit = std::max<int64_t>(rows, (budget - 16 * rows - 1024) / 12);
+    return (int)std::min<int64_t>(std::max<int64_t>(1, max_off) * rows, fit);
+}
+
+// Whether a third CTA per SM saves FP32 sweeps of a mixed cycle a round of tiles:
+// with few tiles a CTA its longer grid barrier and lesser share of the SM are only
+// made good where the SM's last round was not full (8 % short of full at least: a
+// fuller third round is as long).  7-point, cycles of 128, us a sweep with 2 / 3 CTAs:
+// 40^3 (1 round / 1) 3.20 / 3.59, 46^3 (2 / 1) 3.80 / 3.64, 50^3 (2 / 2) 3.88 / 4.26, 52^3 (2 /
+// 2) 3.83 / 4.33, 54^3 (3 / 2) 4.45 / 4.31, 64^3 (4 / 3) 5.46 / 5.32, 68^3 (5 / 3) 6.20 / 5.40;
+// full rounds: 48^3 (2 / 1, 95 % full) 3.78 / 3.80, one cycle alone 526 / 550 us; 5-point
+// 340^2 (2 / 1, 99 %) 3.56 / 3.69.
+static bool third_cta_saves_a_round(const ScaledForm& tf, int sms)
+{
+    const int entries = stage_entries(256, 256, 3, 3, tf.max_off);
+    const double tiles = std::max((double)tf.n / 256.0, (double)tf.rowptr[tf.n] / entries);
+    const double third = tiles / (3.0 * sms);       // rounds of 3 CTAs per SM
+    return std::ceil(1.5 * third) > std::ceil(third + 0.08);
+}
+
 // CTAs per SM and pipeline stages (0: the default 4) where the caller leaves
 // both open.  Measured on GB300, us per sweep without calibration:
 //   one lane per row (7-point), 2 against 3 CTAs/SM: a third CTA hides more of
 //     the gathers' latency and costs a longer grid barrier.  FP64: 64^3 10.7 /
 //     11.8, 128^3 37.3 / 37.3, 160^3 70.2 / 66.1; a mixed cycle's FP32 sweeps
-//     (bound by that latency) from about 100,000 rows on: 48^3 4.03 / 3.98, 96^3
-//     13.0 / 10.6, 128^3 25.9 / 21.3, 160^3 48.2 / 38.9 with cycles of 128 sweeps; its
-//     longer barriers and launches count per cycle, so shorter cycles need more rows
-//     (118x42x22 in boxes, of 32 5.01 / 5.32, of 64 4.19 / 4.40; 64^3, of 32 6.79 /
-//     6.79, of 64 5.95 / 5.81; 100x90x95, of 32 13.2 / 11.9); a split interface block
+//     (bound by that latency), where it saves a round of tiles, from about 100,000
+//     rows on: 64^3 5.46 / 5.32, 80^3 8.18 / 7.22, 96^3 13.0 / 10.6, 128^3 25.9 / 21.3,
+//     160^3 48.2 / 38.9 with cycles of 128 sweeps; its longer barriers and launches
+//     count per cycle, so shorter cycles need more rows (118x42x22 in boxes, of 32 5.01 /
+//     5.32, of 64 4.19 / 4.40; 64^3, of 32 6.48 / 6.37, of 64 5.82 / 5.64; 100x90x95, of
+//     32 13.2 / 11.9; 100^3, of 8 22.8 / 21.6), longer ones fewer (46^3, of 512 3.64 /
+//     3.43; 32^3, of 4096 2.67 / 3.11: no round saved); a split interface block
 //     (slot rows wait longer) from about 1,000,000: 80^3 in 4x4x4 16.4 / 17.2, 104^3
 //     27.4 / 26.6, 128^3 42.6 / 41.2;
 //   the same, FP64, 2 CTAs/SM, 4 / 2 stages: while the matrix comes from L2 two are
@@ -1026,10 +1056,13 @@ static bool fits_l2(int64_t entries, bool mixed) { return (mixed ? 8.0 : 12.0) *
 //     24.5 / 24.3 / 20.7, 128^3 152 / 139 / 127; mixed 48^3 7.1 / 6.6 / 5.8, 64^3
 //     13.6 / 11.7 / 11.5, 96^3 40.7 / 34.7 / 39.0 (FP32 entries take two thirds
 //     of the space, and 36 KB hold the tile).
-static void default_geometry(int lanes, bool mixed, int inner, bool split, int64_t rows, int* per_sm, int* stages)
+static void default_geometry(int lanes, bool mixed, int inner, bool split, const ScaledForm& tf, int sms, int* per_sm,
+                             int* stages)
 {
+    const int64_t rows = tf.n;
     if (lanes == 1) {
-        *per_sm = rows >= (mixed ? 12800000 / std::max(1, inner) : split ? 1000000 : 3000000) ? 3 : 2;
+        if (mixed) *per_sm = rows >= 12800000 / std::max(1, inner) && third_cta_saves_a_round(tf, sms) ? 3 : 2;
+        else *per_sm = rows >= (split ? 1000000 : 3000000) ? 3 : 2;
         if (!mixed && rows < 600000) *stages = 2;
     } else *stages = mixed && rows > 350000 ? 3 : 2;
 }
@@ -1058,18 +1091,6 @@ static int64_t resident_plan(const ScaledForm& tf, const Plan& plan, int ctas, i
         most = std::max(most, b);
     }
     return most;
-}
-
-// Entries that a pipeline stage holds for a tile of `rows` rows: variant 2 has 2
-// CTAs/SM x 4 stages for 224/256-thread tiles (or 3 / 2 larger stages), 3 CTAs/SM x 3
-// stages, 1 CTA/SM x 4 stages for 480-row tiles.
-static int stage_entries(int tile_rows, int rows, int per_sm, int stages, int64_t max_off)
-{
-    int64_t budget = tile_rows <= 256 ? 26 * 1024 : 52 * 1024;
-    if (tile_rows == 256 && per_sm == 2 && stages == 3) budget = 36 * 1024;
-    if (tile_rows == 256 && per_sm == 2 && stages == 2) budget = 54 * 1024;
-    const int64_t fit = std::max<int64_t>(rows, (budget - 16 * rows - 1024) / 12);
-    return (int)std::min<int64_t>(std::max<int64_t>(1, max_off) * rows, fit);
 }
 
 // Sets up the second geometry of a context (per_sm CTAs/SM, stages) for calls of at
@@ -1191,7 +1212,8 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     const bool open = c->variant == 2 && c->rows_per_tile == 256 && !o.ctas_per_sm && !o.stages &&
                       o.sync == JAC_SYNC_GRID && o.stop == JAC_STOP_GLOBAL;
     if (open)
-        default_geometry(c->lanes, o.precision == JAC_MIXED, o.inner_sweeps, sp != nullptr, rows, &target_per_sm, &stages);
+        default_geometry(c->lanes, o.precision == JAC_MIXED, o.inner_sweeps, sp != nullptr, tf, prop.multiProcessorCount,
+                         &target_per_sm, &stages);
     if (target_per_sm == 3) c->stages = 3;
     // fewer, larger stages (2 CTAs/SM, 256 threads): room for whole tiles of long rows
     if (c->variant == 2 && c->rows_per_tile == 256 && target_per_sm == 2 && (stages == 2 || stages == 3))
@@ -1418,7 +1440,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     // 15.0 / 13.6, 128^3 36.7 / 36.6; one sweep alone 100^3 37.0 / 35.5, 128^3 51.4 / 49.8.
     if (open && o.precision == JAC_MIXED && c->variant == 2 && c->lanes == 1 && target_per_sm == 3) {
         int per_sm = 2, fp64_stages = 4;
-        default_geometry(c->lanes, false, o.inner_sweeps, false, rows, &per_sm, &fp64_stages);
+        default_geometry(c->lanes, false, o.inner_sweeps, false, tf, prop.multiProcessorCount, &per_sm, &fp64_stages);
         if (per_sm == 2) {
             st = second_geometry(C, plan, tf, per_sm, fp64_stages, INT32_MAX, nullptr, prop.multiProcessorCount);
             if (st != JAC_OK) return st;

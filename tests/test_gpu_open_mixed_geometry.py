@@ -1,0 +1,45 @@
+"""The geometry that an open jac_opts gives mixed contexts, on both sides of the
+sizes where it changes, against a pinned one: whole cycles bit for bit (an FP32
+sweep's sums do not depend on tiles or CTAs, and its FP64 pass keeps each row's).
+
+Test values: both add the same n squares, in different orders, so each sum
+carries at most n roundings of it: relative difference <= 2 n u."""
+import numpy as np
+import pytest
+
+from paper_2112_02377_gb300 import jacobi as J
+from paper_2112_02377_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+def _check(A, per_sm, stages, inner, split=J.JAC_BANDROW, **kw):
+    b = np.random.default_rng(1).uniform(-1, 1, A.n)
+    kw.update(precision=J.JAC_MIXED, inner_sweeps=inner)
+    a = J.jac_setup(A, b, split, 3, J.opts(**kw))
+    s = J.jac_stats(a)
+    other = 2 if per_sm == 3 else 3
+    p = J.jac_setup(A, b, split, 3, J.opts(lanes_per_row=s["lanes_per_row"], variant=2, ctas_per_sm=other, **kw))
+    try:
+        assert (s["ctas_per_sm"], s["stages"]) == (per_sm, stages)
+        for _ in range(2):
+            k = J.jac_stats(a)["k"] + 2 * inner
+            ra, rp = J.jac_solve(a, 1e-30, k), J.jac_solve(p, 1e-30, k)
+            assert ra[0] == rp[0] and ra[2] == rp[2] and abs(ra[1] - rp[1]) <= 2 * A.n * U * rp[1]
+            assert np.array_equal(J.jac_get_x(a, None, A.n), J.jac_get_x(p, None, A.n))
+    finally:
+        J.jac_free(a)
+        J.jac_free(p)
+
+
+@pytest.mark.parametrize("dims,inner,per_sm", [
+    ((50, 50, 50), 128, 2),                   # 2 rounds of tiles with two CTAs per SM, 2 with three
+    ((54, 54, 54), 128, 3),                   # 3 and 2
+    ((48, 48, 48), 128, 2),                   # 2 and 1, the one 95 % full
+    ((47, 47, 48), 128, 3),                   # 2 and 1, 91 %
+    ((46, 46, 46), 128, 2), ((46, 46, 46), 132, 3),      # rows times the cycle's sweeps
+    ((16, 16, 16), 4096, 2), ((40, 40, 40), 512, 2),     # long cycles, one round either way
+    ((74, 73, 74), 32, 2), ((74, 74, 74), 32, 3)])       # short ones
+def test_open_mixed_geometry_one_lane(dims, inner, per_sm):
+    _check(W.laplace7(dims), per_sm, 3 if per_sm == 3 else 4, inner)
