@@ -1034,6 +1034,23 @@ static bool third_cta_saves_a_round(const ScaledForm& tf, int sms)
     return std::ceil(1.5 * third) > std::ceil(third + 0.08);
 }
 
+// Stretches of the iterate (columns at most 8 apart) that a row reads, on average over
+// up to 1,024 rows: 3 in a plane's 5- or 9-point operator, 5 and 9 in space.  A tile's
+// rows read the same stretches side by side, so with few of them the gathers find
+// their lines in L1 and there is little latency for a third CTA to hide.
+static double gather_stretches(const ScaledForm& tf)
+{
+    const int64_t step = std::max<int64_t>(1, tf.n / 1024);
+    int64_t rows = 0, stretches = 0;
+    std::vector<int32_t> col;
+    for (int64_t r = step / 2; r < tf.n; r += step, ++rows) {
+        col.assign(tf.col.begin() + tf.rowptr[r], tf.col.begin() + tf.rowptr[r + 1]);
+        std::sort(col.begin(), col.end());
+        for (size_t k = 0; k < col.size(); ++k) stretches += k == 0 || col[k] - col[k - 1] > 8;
+    }
+    return rows ? (double)stretches / (double)rows : 0.0;
+}
+
 // CTAs per SM and pipeline stages (0: the default 4) where the caller leaves
 // both open.  Measured on GB300, us per sweep without calibration:
 //   one lane per row (7-point), 2 against 3 CTAs/SM: a third CTA hides more of
@@ -1045,7 +1062,12 @@ static bool third_cta_saves_a_round(const ScaledForm& tf, int sms)
 //     count per cycle, so shorter cycles need more rows (118x42x22 in boxes, of 32 5.01 /
 //     5.32, of 64 4.19 / 4.40; 64^3, of 32 6.48 / 6.37, of 64 5.82 / 5.64; 100x90x95, of
 //     32 13.2 / 11.9; 100^3, of 8 22.8 / 21.6), longer ones fewer (46^3, of 512 3.64 /
-//     3.43; 32^3, of 4096 2.67 / 3.11: no round saved); a split interface block
+//     3.43; 32^3, of 4096 2.67 / 3.11: no round saved).  Rows that read fewer than four
+//     stretches of the iterate gain later: 5-point 400^2 4.16 / 4.28, 600^2 5.62 / 6.02,
+//     700^2 6.99 / 6.96, 800^2 8.49 / 7.92; 9-point 500^2 6.62 / 6.98, 800^2 13.28 / 13.43,
+//     1000^2 19.4 / 19.0 (from 120,000 rows an entry on), and 9-point ones not at all in
+//     FP64: 1800^2 80.6 / 82.1, 2100^2 108.3 / 110.1 (5-point 46.1 / 42.8, 72.7 [2200^2] /
+//     62.2).  A split interface block
 //     (slot rows wait longer) from about 1,000,000: 80^3 in 4x4x4 16.4 / 17.2, 104^3
 //     27.4 / 26.6, 128^3 42.6 / 41.2;
 //   the same, FP64, 2 CTAs/SM, 4 / 2 stages: while the matrix comes from L2 two are
@@ -1061,8 +1083,15 @@ static void default_geometry(int lanes, bool mixed, int inner, bool split, const
 {
     const int64_t rows = tf.n;
     if (lanes == 1) {
-        if (mixed) *per_sm = rows >= 12800000 / std::max(1, inner) && third_cta_saves_a_round(tf, sms) ? 3 : 2;
-        else *per_sm = rows >= (split ? 1000000 : 3000000) ? 3 : 2;
+        const double entries = (double)tf.rowptr[rows] / (double)std::max<int64_t>(1, rows);
+        auto compact = [&] { return !split && gather_stretches(tf) < 4.0; };
+        bool third;
+        if (mixed)
+            third = rows >= 12800000 / std::max(1, inner) && third_cta_saves_a_round(tf, sms) &&
+                    ((double)rows >= 120000.0 * entries || !compact());
+        else
+            third = rows >= (split ? 1000000 : 3000000) && !(entries > 6.0 && compact());
+        *per_sm = third ? 3 : 2;
         if (!mixed && rows < 600000) *stages = 2;
     } else *stages = mixed && rows > 350000 ? 3 : 2;
 }

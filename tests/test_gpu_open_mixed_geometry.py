@@ -43,3 +43,38 @@ def _check(A, per_sm, stages, inner, split=J.JAC_BANDROW, **kw):
     ((74, 73, 74), 32, 2), ((74, 74, 74), 32, 3)])       # short ones
 def test_open_mixed_geometry_one_lane(dims, inner, per_sm):
     _check(W.laplace7(dims), per_sm, 3 if per_sm == 3 else 4, inner)
+
+
+def _plane(edge, corners):
+    """A plane's 5- or 9-point operator on edge x edge nodes (diagonal 4 or 8, others -1)."""
+    n = edge * edge
+    i, j = np.arange(n) % edge, np.arange(n) // edge
+    offs = [(a, c) for c in (-1, 0, 1) for a in (-1, 0, 1) if corners or a == 0 or c == 0]
+    ok = np.stack([(i + a >= 0) & (i + a < edge) & (j + c >= 0) & (j + c < edge) for a, c in offs], 1)
+    col = np.stack([i + a + edge * (j + c) for a, c in offs], 1)
+    val = np.tile([float(len(offs) - 1) if a == c == 0 else -1.0 for a, c in offs], (n, 1))
+    ptr = np.concatenate([[0], np.cumsum(ok.sum(1))])
+    return W.CSR(n=n, rowptr=ptr.astype(np.int32), col=col[ok].astype(np.int32), val=val[ok])
+
+
+@pytest.mark.parametrize("edge,corners,per_sm", [(450, False, 2), (700, False, 3), (500, True, 2), (980, True, 3)])
+def test_open_mixed_geometry_of_planes(edge, corners, per_sm):
+    _check(_plane(edge, corners), per_sm, 3 if per_sm == 3 else 4, 128)
+
+
+@pytest.mark.parametrize("corners,per_sm,stages", [(False, 3, 3), (True, 2, 4)])
+def test_open_fp64_geometry_of_planes(corners, per_sm, stages):
+    A = _plane(1740, corners)                 # 3,027,600 rows
+    b = np.random.default_rng(2).uniform(-1, 1, A.n)
+    a = J.jac_setup(A, b, J.JAC_BANDROW, 1, J.opts())
+    p = J.jac_setup(A, b, J.JAC_BANDROW, 1, J.opts(variant=2, ctas_per_sm=5 - per_sm))
+    try:
+        s = J.jac_stats(a)
+        assert (s["ctas_per_sm"], s["stages"]) == (per_sm, stages)
+        for k in (1, 6):
+            ra, rp = J.jac_sweep(a, k), J.jac_sweep(p, k)
+            assert np.array_equal(J.jac_get_x(a, None, A.n), J.jac_get_x(p, None, A.n))
+            assert abs(ra - rp) <= 2 * A.n * U * rp
+    finally:
+        J.jac_free(a)
+        J.jac_free(p)
