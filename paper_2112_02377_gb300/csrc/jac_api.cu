@@ -1467,10 +1467,13 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     // CTA per SM, which those sweeps do not: they take an FP64 context's geometry.
     // us a sweep in the cycles' / there: 7-point 48^3 8.8 / 7.3, 64^3 11.1 / 9.9, 80^3
     // 15.0 / 13.6, 128^3 36.7 / 36.6; one sweep alone 100^3 37.0 / 35.5, 128^3 51.4 / 49.8.
+    // Rows of more than eight entries, of which four small stages hold too few at a
+    // time, stay with the third CTA where two large ones are not to be had: 15-point
+    // 76^3 21.7 / 18.1, 90^3 31.3 / 35.6, 100^3 38.7 / 47.2.
     if (open && o.precision == JAC_MIXED && c->variant == 2 && c->lanes == 1 && target_per_sm == 3) {
         int per_sm = 2, fp64_stages = 4;
         default_geometry(c->lanes, false, o.inner_sweeps, false, tf, prop.multiProcessorCount, &per_sm, &fp64_stages);
-        if (per_sm == 2) {
+        if (per_sm == 2 && (fp64_stages == 2 || nnz_off <= 8 * rows)) {
             st = second_geometry(C, plan, tf, per_sm, fp64_stages, INT32_MAX, nullptr, prop.multiProcessorCount);
             if (st != JAC_OK) return st;
         }

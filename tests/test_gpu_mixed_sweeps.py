@@ -35,3 +35,29 @@ def test_fp64_sweeps_of_a_mixed_context(dims, split, per_sm):
             assert np.array_equal(a.x(), p.x())
             a.sweep(3), p.sweep(3)
             assert np.array_equal(a.x(), p.x())
+
+
+def _fifteen_points(edge):
+    """The faces' and corners' neighbours on edge^3 nodes (diagonal 14, others -1)."""
+    n = edge ** 3
+    g = np.arange(n)
+    node = (g % edge, g // edge % edge, g // edge ** 2)
+    offs = [(a, c, e) for e in (-1, 0, 1) for c in (-1, 0, 1) for a in (-1, 0, 1) if abs(a) + abs(c) + abs(e) in (0, 1, 3)]
+    ok = np.stack([np.all([(node[q] + o[q] >= 0) & (node[q] + o[q] < edge) for q in range(3)], axis=0) for o in offs], 1)
+    col = np.stack([g + o[0] + edge * (o[1] + edge * o[2]) for o in offs], 1)
+    val = np.tile([14.0 if o == (0, 0, 0) else -1.0 for o in offs], (n, 1))
+    ptr = np.concatenate([[0], np.cumsum(ok.sum(1))])
+    return W.CSR(n=n, rowptr=ptr.astype(np.int32), col=col[ok].astype(np.int32), val=val[ok])
+
+
+@pytest.mark.parametrize("edge,per_sm", [(60, 2), (86, 3)])    # two large stages below 600,000 rows
+def test_fp64_sweeps_of_longer_rows(edge, per_sm):
+    A = _fifteen_points(edge)
+    b = np.random.default_rng(8).uniform(-1, 1, A.n)
+    with J.Solver(A, b, precision=J.JAC_MIXED) as a, J.Solver(A, b, variant=2, ctas_per_sm=2, lanes_per_row=1) as f:
+        sms = a.stats()["ctas"] // 3
+        assert a.stats()["ctas_per_sm"] == 3
+        for k in (1, 4):
+            ra, rf = a.sweep(k), f.sweep(k)
+            assert len(J.jac_get_trace(a.ctx)[0]) == per_sm * sms
+            assert np.array_equal(a.x(), f.x()) and abs(ra - rf) <= 2 * A.n * U * rf
