@@ -1077,7 +1077,11 @@ static double gather_stretches(const ScaledForm& tf)
 //     rows of a two-lane tile, a 54 KB one all.  FP64: 32^3 9.6 / 9.5 / 8.6, 64^3
 //     24.5 / 24.3 / 20.7, 128^3 152 / 139 / 127; mixed 48^3 7.1 / 6.6 / 5.8, 64^3
 //     13.6 / 11.7 / 11.5, 96^3 40.7 / 34.7 / 39.0 (FP32 entries take two thirds
-//     of the space, and 36 KB hold the tile).
+//     of the space, and 36 KB hold the tile).  Four and eight lanes, FP64: 45-point 72^3
+//     54.0 / 52.8 / 48.2, 125-point 64^3 117 / 97 / 89; mixed 45-point 64^3 20.6 / 18.5 /
+//     19.2, 125-point 48^3 24.7 / 22.4 / 21.5, 64^3 56.0 / 50.7 / 47.9; but 75-point rows,
+//     whose tiles of 32 nearly fit a small stage, mixed, past L2: 56^3 22.7 / 22.4 / 23.8,
+//     64^3 33.3 / 34.0 / 35.8, 84^3 70.2 / 71.2 / 75.5 (48^3, in L2, 14.1 / 14.3 / 13.7).
 static void default_geometry(int lanes, bool mixed, int inner, bool split, const ScaledForm& tf, int sms, int* per_sm,
                              int* stages)
 {
@@ -1093,7 +1097,12 @@ static void default_geometry(int lanes, bool mixed, int inner, bool split, const
             third = rows >= (split ? 1000000 : 3000000) && !(entries > 6.0 && compact());
         *per_sm = third ? 3 : 2;
         if (!mixed && rows < 600000) *stages = 2;
-    } else *stages = mixed && rows > 350000 ? 3 : 2;
+    } else {
+        *stages = mixed && rows > 350000 ? 3 : 2;
+        const double tile = 256.0 / lanes * (double)tf.rowptr[rows] / (double)std::max<int64_t>(1, rows);
+        if (mixed && lanes == 8 && !fits_l2(tf.rowptr[rows], true) && 7.0 * tile <= 8.0 * stage_entries(256, 32, 2, 4, INT32_MAX / 32))
+            *stages = 4;
+    }
 }
 
 // Row ranges of the resident kernel's CTAs and the dynamic shared memory of the

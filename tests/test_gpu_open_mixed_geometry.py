@@ -78,3 +78,28 @@ def test_open_fp64_geometry_of_planes(corners, per_sm, stages):
     finally:
         J.jac_free(a)
         J.jac_free(p)
+
+
+def _box_rows(edge, reach):
+    """Every node of a box of +-reach around a node of edge^3 (diagonal the entries less one, others -1)."""
+    n = edge ** 3
+    g = np.arange(n)
+    node = (g % edge, g // edge % edge, g // edge ** 2)
+    offs = [(a, c, e) for e in range(-reach[2], reach[2] + 1) for c in range(-reach[1], reach[1] + 1)
+            for a in range(-reach[0], reach[0] + 1)]
+    ok = np.stack([np.all([(node[q] + o[q] >= 0) & (node[q] + o[q] < edge) for q in range(3)], axis=0) for o in offs], 1)
+    col = np.stack([g + o[0] + edge * (o[1] + edge * o[2]) for o in offs], 1)
+    val = np.tile([float(len(offs) - 1) if o == (0, 0, 0) else -1.0 for o in offs], (n, 1))
+    ptr = np.concatenate([[0], np.cumsum(ok.sum(1))])
+    return W.CSR(n=n, rowptr=ptr.astype(np.int32), col=col[ok].astype(np.int32), val=val[ok])
+
+
+@pytest.mark.parametrize("edge,reach,lanes,stages", [
+    (48, (1, 2, 2), 8, 2), (54, (1, 2, 2), 8, 4),     # 75-point rows, in L2 and past it
+    (48, (2, 2, 2), 8, 2),                            # 125-point rows
+    (70, (1, 1, 1), 2, 2), (71, (1, 1, 1), 2, 3)])    # 27-point rows on both sides of 350,000
+def test_open_mixed_geometry_several_lanes(edge, reach, lanes, stages):
+    A = _box_rows(edge, reach)
+    with J.Solver(A, None, precision=J.JAC_MIXED) as s:
+        assert s.stats()["lanes_per_row"] == lanes
+    _check(A, 2, stages, 32)
