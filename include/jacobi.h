@@ -129,8 +129,8 @@ typedef struct {
 typedef struct {
     int32_t precision;         /* jac_precision (default JAC_FP64) */
     int32_t norm;              /* jac_norm (default JAC_NORM_REL2) */
-    int32_t sweeps_per_graph;  /* sweeps per CUDA-graph launch, 1..4096 (default 64; at least 512 where the
-                                  matrix is kept in shared memory, see variant) */
+    int32_t sweeps_per_graph;  /* sweeps per CUDA-graph launch, 1..4096 (default 64, which stands for 512
+                                  where the matrix is kept in shared memory, see variant) */
     int32_t inner_sweeps;      /* JAC_MIXED: FP32 sweeps per FP64 refinement step, >= 1 (default 128) */
     int32_t grid[3];           /* node grid (gx, gy, gz); required for JAC_SUBSTRUCT */
     int32_t subdomains[3];     /* boxes per axis (px, py, pz); JAC_SUBSTRUCT only */

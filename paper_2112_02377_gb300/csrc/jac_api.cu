@@ -417,10 +417,8 @@ int mixed_cycles_per_step(const jac_ctx* c)
     return std::max(1, (c->K + m - 1) / m);
 }
 
-// FP64 sweeps of a graph step.  The resident kernel loads the matrix and ends
-// with a barrier of its own in every launch (3 to 9 us together), against 2 us
-// a sweep: its steps have at least 512 sweeps.
-int sweeps_per_step(const jac_ctx* c) { return c->resident ? std::max(c->K, 512) : c->K; }
+// FP64 sweeps of a graph step.
+int sweeps_per_step(const jac_ctx* c) { return c->resident ? resident_step(c->K) : c->K; }
 
 // Sweeps whose per-set maxima are kept (local stopping).
 int loc_slots(const jac_ctx* c) { return c->resident ? 4 : 3; }
@@ -1269,6 +1267,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
         const void* fn = resident_kernel(c->lanes, local_stop);
         if (need > 0 && need <= (int64_t)prop.sharedMemPerBlockOptin && coop &&
+            resident_step(c->K) > resident_short_calls(need) &&
             allow_smem(fn, (int)need) == cudaSuccess &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, fn, resident_threads(), (size_t)need) == cudaSuccess &&
             fits >= 1) {

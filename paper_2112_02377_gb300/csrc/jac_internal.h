@@ -18,6 +18,11 @@ inline bool usable_in_place(bool device_memory, int owner, int device, uintptr_t
     return device_memory && owner == device && (p & 7u) == 0;
 }
 
+// Sweeps of a launch of the resident kernel: what the caller asks for; the default of
+// 64 stands for 512 there, as every launch loads the matrix and ends with a barrier of
+// its own (3 to 9 us together, against 2 to 7 us a sweep).
+inline int resident_step(int sweeps_per_graph) { return sweeps_per_graph == 64 ? 512 : sweeps_per_graph; }
+
 // A square matrix in 0-based CSR, host memory.
 struct HostCSR {
     int64_t n = 0;
