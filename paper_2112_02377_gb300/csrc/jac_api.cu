@@ -36,7 +36,8 @@ struct SecondGeometry {
     const void* fn = nullptr;      // nullptr: none
     int64_t most = 0;              // sweeps of the longest call that runs in it
     int grid = 0, threads = 0, smem = 0, ntiles = 0, emax = 0;
-    int *d_row0 = nullptr, *d_nnz0 = nullptr, *d_cta0 = nullptr;
+    std::vector<int32_t> tables;   // row0, nnz0 (ntiles+1 each) and cta0 (grid+1) until they are on the device
+    int* d_tables = nullptr;
 };
 
 struct jac_ctx {
@@ -376,11 +377,11 @@ DevTiles second_tiles(const jac_ctx* c)
 {
     const SecondGeometry& g = c->second;
     DevTiles t{};
-    t.row0 = g.d_row0;
-    t.nnz0 = g.d_nnz0;
-    t.row1 = g.d_row0 + 1;
-    t.nnz1 = g.d_nnz0 + 1;
-    t.cta0 = g.d_cta0;
+    t.row0 = g.d_tables;
+    t.nnz0 = t.row0 + g.ntiles + 1;
+    t.row1 = t.row0 + 1;
+    t.nnz1 = t.nnz0 + 1;
+    t.cta0 = t.nnz0 + g.ntiles + 1;
     t.ntiles = g.ntiles;
     t.keep = c->keep_l2 ? 1 : 0;
     t.emax = g.emax;
@@ -491,9 +492,11 @@ jac_status second_step(jac_ctx* c, int64_t sweeps)
 {
     cudaStream_t s = stream_of(c);
     const SecondGeometry& g = c->second;
+    DevVec v = devvec(c);
+    v.nslots = g.grid;
     for (int64_t left = sweeps; left > 0; left -= c->K) {
         CK(c, launch_reset_bar(c->d_ctl, s));
-        CK(c, launch_persistent(g.fn, g.grid, g.threads, g.smem, devmat(c), devvec(c), second_tiles(c), c->d_ctl,
+        CK(c, launch_persistent(g.fn, g.grid, g.threads, g.smem, devmat(c), v, second_tiles(c), c->d_ctl,
                                 (int)std::min<int64_t>(left, c->K), s));
     }
     return JAC_OK;
@@ -619,7 +622,7 @@ jac_status status_from_ctl(jac_ctx* c, const JacCtl& h)
 jac_status arm(jac_ctx* c, int test, int mixed, long long k_limit, long long k_delta, double tol)
 {
     if (c->d_trace)
-        CK(c, cudaMemsetAsync(c->d_trace, 0, 4 * sizeof(unsigned long long) * c->nslots, stream_of(c)));
+        CK(c, cudaMemsetAsync(c->d_trace, 0, 4 * sizeof(unsigned long long) * std::max(c->grid, c->second.grid), stream_of(c)));
     if (c->d_loc)
         CK(c, cudaMemsetAsync(c->d_loc, 0, loc_slots(c) * sizeof(unsigned long long) * c->nloc, stream_of(c)));
     CK(c, launch_arm(c->d_ctl, test, mixed, c->o.inner_sweeps, k_limit, k_delta, tol, c->o.norm, c->d_hist, c->hist_cap,
@@ -647,7 +650,7 @@ void destroy(jac_ctx* c)
     dfree(c->d_rowptr); dfree(c->d_col); dfree(c->d_S64); dfree(c->d_S32); dfree(c->d_b); dfree(c->d_d);
     dfree(c->d_x[0]); dfree(c->d_x[1]); dfree(c->d_x[2]); dfree(c->d_x[3]); dfree(c->d_x[4]);
     dfree(c->d_cta_row);
-    dfree(c->second.d_row0); dfree(c->second.d_nnz0); dfree(c->second.d_cta0);
+    dfree(c->second.d_tables);
     dfree(c->d_dep_ptr); dfree(c->d_dep); dfree(c->d_done); dfree(c->d_e[0]); dfree(c->d_e[1]); dfree(c->d_dlt);
     dfree(c->d_part); dfree(c->d_ctl); dfree(c->d_hist); dfree(c->d_perm); dfree(c->d_stage); dfree(c->d_stage2);
     dfree(c->d_bmap); dfree(c->d_slot_info);
@@ -987,10 +990,14 @@ inline int64_t nnz_off_of(const ScaledForm& tf) { return tf.rowptr.empty() ? 0 :
 // rows have 11 to 17 entries instead of 26, put the own work at 19 entries in FP64
 // and 50 in mixed cycles, whose FP32 sweeps are bound by the latency of a row's
 // rounds of gathers and not by its entries (96^3 FP64 57.6 -> 54.1 us a sweep, 61^3
-// mixed 10.0 -> 9.2: the first and last CTAs had a third more rows).  Rows of a
-// substructuring's interface gather from several subdomains: their CTAs took
-// 17 % longer in mixed cycles (131x128x125 in 4x4x4: 22.9 -> 21.6 us); smaller systems
-// gain nothing from it (FP64 sweeps of 100x90x95 1 % slower): from 1,500,000 rows on.
+// mixed 10.0 -> 9.2: the first and last CTAs had a third more rows; four and eight
+// lanes, 45-point 72^3 FP64 52.1 -> 48.2, 125-point 64^3 91.9 -> 88.9, mixed 55.3 -> 48.6).
+// Rows of a substructuring's interface gather from several subdomains: their CTAs
+// took 17 % longer in mixed cycles.  us a sweep of those without / with that, boxes 2x2x2,
+// 4x4x4, 8x8x8: 70^3 5.85 / 5.68, 5.90 / 6.10, 6.21 / 6.32; 96^3 10.21 / 9.93, 10.13 / 10.13,
+// 10.41 / 10.42; 120^3 18.7 / 18.3, 18.5 / 18.3, 18.5 / 18.7; 131x128x125 22.8 / 21.5,
+// 22.8 / 21.5, 21.9 / 22.0; 140^3 28.3 / 26.7, 28.1 / 26.8, 27.9 / 27.8.  Small systems in many
+// boxes lose what those in few gain: from 1,500,000 rows on.
 static double form_row_cost(int64_t len, int lanes, bool mixed, bool interface_row)
 {
     if (lanes > 1) return (mixed ? 50.0 : 19.0) + (double)len;
@@ -1131,8 +1138,8 @@ static int64_t resident_plan(const ScaledForm& tf, const Plan& plan, int ctas, i
 
 // Sets up the second geometry of a context (per_sm CTAs/SM, stages) for calls of at
 // most `most` FP64 sweeps; where it cannot be had every call keeps the first.
-static jac_status second_geometry(jac_ctx* c, const Plan& plan, const ScaledForm& tf, int per_sm, int stages, int64_t most,
-                                  const std::vector<double>* row_cost, int sms)
+static void second_geometry(jac_ctx* c, const Plan& plan, const ScaledForm& tf, int per_sm, int stages, int64_t most,
+                            const std::vector<double>* row_cost, int sms)
 {
     const int rows = 256 / c->lanes;
     SecondGeometry g;
@@ -1145,27 +1152,15 @@ static jac_status second_geometry(jac_ctx* c, const Plan& plan, const ScaledForm
     if (!fn || allow_smem(fn, g.smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, fn, g.threads, g.smem) != cudaSuccess || fits < 1) {
         cudaGetLastError();
-        return JAC_OK;
+        return;
     }
     g.grid = std::min(fits, per_sm) * sms;
     Tiling t;
     make_tiling(tf, plan, rows, g.emax, g.grid, t, row_cost);
     g.ntiles = (int)t.ntiles();
-    auto upload = [&](int** d, const std::vector<int32_t>& v) -> jac_status {
-        CK(nullptr, dalloc(d, v.size()));
-        CK(nullptr, cudaMemcpy(*d, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-        return JAC_OK;
-    };
-    jac_status st = upload(&c->second.d_row0, t.row0);
-    if (st == JAC_OK) st = upload(&c->second.d_nnz0, t.nnz0);
-    if (st == JAC_OK) st = upload(&c->second.d_cta0, t.cta0);
-    if (st != JAC_OK) return st;
-    g.d_row0 = c->second.d_row0;
-    g.d_nnz0 = c->second.d_nnz0;
-    g.d_cta0 = c->second.d_cta0;
     g.fn = fn;
-    c->second = g;
-    return JAC_OK;
+    for (const auto* v : {&t.row0, &t.nnz0, &t.cta0}) g.tables.insert(g.tables.end(), v->begin(), v->end());
+    c->second = std::move(g);
 }
 
 // Sweeps of the longest call that the resident kernel loses to the pipelined one: a
@@ -1467,9 +1462,8 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
             est_cost.resize(rows);
             for (int64_t r = 0; r < rows; ++r) est_cost[r] = form_row_cost(tf.rowptr[r + 1] - tf.rowptr[r], c->lanes, false, false);
         }
-        st = second_geometry(C, plan, tf, target_per_sm, pipelined_stages, short_calls,
-                             est_cost.empty() ? nullptr : &est_cost, prop.multiProcessorCount);
-        if (st != JAC_OK) return st;
+        second_geometry(C, plan, tf, target_per_sm, pipelined_stages, short_calls,
+                        est_cost.empty() ? nullptr : &est_cost, prop.multiProcessorCount);
     }
     // FP64 sweeps of a mixed context (jac_sweep) whose cycles run best with a third
     // CTA per SM, which those sweeps do not: they take an FP64 context's geometry.
@@ -1481,12 +1475,10 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
     if (open && o.precision == JAC_MIXED && c->variant == 2 && c->lanes == 1 && target_per_sm == 3) {
         int per_sm = 2, fp64_stages = 4;
         default_geometry(c->lanes, false, o.inner_sweeps, false, tf, prop.multiProcessorCount, &per_sm, &fp64_stages);
-        if (per_sm == 2 && (fp64_stages == 2 || nnz_off <= 8 * rows)) {
-            st = second_geometry(C, plan, tf, per_sm, fp64_stages, INT32_MAX, nullptr, prop.multiProcessorCount);
-            if (st != JAC_OK) return st;
-        }
+        if (per_sm == 2 && (fp64_stages == 2 || nnz_off <= 8 * rows))
+            second_geometry(C, plan, tf, per_sm, fp64_stages, INT32_MAX, nullptr, prop.multiProcessorCount);
     }
-    c->nslots = std::max(c->grid, c->second.grid);
+    c->nslots = c->grid;
 
     // ---- device buffers
     CK(nullptr, dalloc(&c->d_rowptr, rows + 1 + 16));
@@ -1524,7 +1516,7 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         CK(nullptr, dalloc(&c->d_e[1], n + 16));
         CK(nullptr, dalloc(&c->d_dlt, n + 16));
     }
-    CK(nullptr, dalloc(&c->d_part, (c->resident ? 4 : 2) * (size_t)c->nslots + 4 + 2));
+    CK(nullptr, dalloc(&c->d_part, std::max((c->resident ? 4 : 2) * (size_t)c->nslots, 2 * (size_t)c->second.grid) + 4 + 2));
     if (c->stop == JAC_STOP_LOCAL) {
         std::vector<int32_t> mem_ptr, mem_part, mem_head;
         const Error el = local_row_sets(plan, o, mem_ptr, mem_part, mem_head, c->h_set_id);
@@ -1541,7 +1533,12 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
             CK(nullptr, cudaMemcpy(c->d_mem_part, mem_part.data(), mem_part.size() * 4, cudaMemcpyHostToDevice));
         CK(nullptr, cudaMemset(c->d_loc, 0, loc_slots(c.get()) * sizeof(unsigned long long) * c->nloc));
     }
-    if (c->variant >= 2) CK(nullptr, dalloc(&c->d_trace, 4 * (size_t)c->nslots));
+    if (c->variant >= 2) CK(nullptr, dalloc(&c->d_trace, 4 * (size_t)std::max(c->grid, c->second.grid)));
+    if (SecondGeometry& g = c->second; g.fn) {
+        CK(nullptr, dalloc(&g.d_tables, g.tables.size()));
+        CK(nullptr, cudaMemcpy(g.d_tables, g.tables.data(), g.tables.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        g.tables = std::vector<int32_t>();
+    }
     CK(nullptr, dalloc(&c->d_ctl, 1));
     CK(nullptr, dalloc(&c->d_stage, n + 16));
     CK(nullptr, cudaMallocHost((void**)&c->h_ctl, 2 * sizeof(JacCtl)));
@@ -1858,11 +1855,12 @@ try {
             jac_free(probe);
         }
     }
-    // The cost model's prior: one lane per row with 3 CTAs/SM and 3 stages
-    // (short rows, FP64-pipe and gather bound); long rows (2+ lanes) with
-    // 2 CTAs/SM and 2 large stages that hold whole tiles of 256/L rows.
+    // The cost model's prior.  FP64 systems of up to 3,000,000 entries: what an open
+    // geometry gives, the resident kernel where the matrix fits and default_geometry's
+    // choice where it does not.  Else one lane per row with 3 CTAs/SM and 3 stages
+    // (short rows, FP64-pipe and gather bound), long rows (2+ lanes) with 2 CTAs/SM and
+    // 2 large stages that hold whole tiles of 256/L rows.
     std::vector<Geometry> cand;
-    // (FP64 systems that fit the chip's shared memory: what an open geometry gives, the resident kernel)
     if (o.precision == JAC_FP64 && !async && resident_kernel(la, local_stop) && !o.stages &&
         prep.tf.rowptr[prep.tf.n] <= 3000000)
         cand.push_back({0, 0, 0, 0});

@@ -96,8 +96,8 @@ __device__ __forceinline__ void block_sums(double& ss, double& mx, double& bb)
         }
 }
 
-// Entries staged at a time: a block's 256 rows of up to 7 entries in one
-// round (21.5 KB, eight blocks an SM); longer rows take several rounds.
+// Entries staged at a time: a block's 256 rows of up to 7 entries in one round (21.5
+// KB; registers, not this, hold an SM to five blocks); longer rows take several rounds.
 constexpr int kCap = 7 * kBlock;
 constexpr int kGather = 7;   // x loads of a row issued together
 

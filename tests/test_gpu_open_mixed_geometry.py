@@ -80,6 +80,11 @@ def test_open_fp64_geometry_of_planes(corners, per_sm, stages):
         J.jac_free(p)
 
 
+@pytest.mark.parametrize("edge", [111, 113, 114, 115])     # entries kept in L2 or not; interface rows cost more from 1,500,000
+def test_open_mixed_geometry_of_boxes(edge):
+    _check(W.laplace7(edge), 3, 3, 32, J.JAC_SUBSTRUCT, grid=(edge,) * 3, subdomains=(2, 2, 2))
+
+
 def _box_rows(edge, reach):
     """Every node of a box of +-reach around a node of edge^3 (diagonal the entries less one, others -1)."""
     n = edge ** 3
