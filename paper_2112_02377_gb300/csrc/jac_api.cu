@@ -1534,13 +1534,13 @@ static jac_status setup_core(const Plan& plan, const ScaledForm& tf, int64_t n, 
         CK(nullptr, cudaMemset(c->d_loc, 0, loc_slots(c.get()) * sizeof(unsigned long long) * c->nloc));
     }
     if (c->variant >= 2) CK(nullptr, dalloc(&c->d_trace, 4 * (size_t)std::max(c->grid, c->second.grid)));
+    CK(nullptr, dalloc(&c->d_ctl, 1));
+    CK(nullptr, dalloc(&c->d_stage, n + 16));
     if (SecondGeometry& g = c->second; g.fn) {
         CK(nullptr, dalloc(&g.d_tables, g.tables.size()));
         CK(nullptr, cudaMemcpy(g.d_tables, g.tables.data(), g.tables.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
         g.tables = std::vector<int32_t>();
     }
-    CK(nullptr, dalloc(&c->d_ctl, 1));
-    CK(nullptr, dalloc(&c->d_stage, n + 16));
     CK(nullptr, cudaMallocHost((void**)&c->h_ctl, 2 * sizeof(JacCtl)));
     std::memset(c->h_ctl, 0, 2 * sizeof(JacCtl));
     if (o.history > 0) {
