@@ -15,14 +15,15 @@
 //   sweep s + 2  a spare warp of CTA 0 adds all CTAs' partials (the barrier of
 //                sweep s + 1 made them visible), takes the decision of sweep s and
 //                publishes it as one word;
-//   sweep s + 3  every CTA reads that word before it arrives at the barrier.
+//   sweep s + 3  every CTA reads that word before it arrives at the barrier, or
+//                already in sweep s + 2 where that is longer than the decision takes.
 // The iterate rotates through five buffers, so the x^k that a stop returns is
 // still there three sweeps later.  Iterates and infinity norms are those of the other
 // kernels bit for bit; 2-norms are the same squares added in another order (2 n u
 // apart at most), so a solve stops in the same sweep unless its test value lies that
-// close to the tolerance.  The price of the late decision is three more sweeps after the
-// one that passes: a solve that its first iterate ends takes 82 us at 70^3, 59 in the
-// pipelined kernel, and is even after about four sweeps.
+// close to the tolerance.  The price of the late decision is two or three more sweeps
+// after the one that passes: a solve that its first iterate ends takes 70 us at 70^3 (82
+// with three), 59 in the pipelined kernel, and is even after two or three sweeps.
 //
 // Measured on GB300, 16^3 7-point: 2.3 to 2.4 us a sweep, of them 1.2 us in the grid
 // barrier (a bare one takes 1.4 us; splitting its counter over several lines or
@@ -221,7 +222,7 @@ long long resident_smem_bytes(const int* rowptr, int r0, int r1, int lanes)
 // the atomics and, where a warp's rows lie in several boxes, finding the peers.
 template <int L, bool LOC>
 __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const int* __restrict__ cta_row, JacCtl* ctl,
-                                                    int max_sweeps)
+                                                    int max_sweeps, int late)
 {
     constexpr int SYNC = (MW + 1) * 32;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -460,12 +461,12 @@ __global__ void __launch_bounds__(RT, 1) k_resident(DevMat m, DevVec v, const in
             }
         } else {
             if (s >= 1) publish_sweep(s - 1);
-            // every CTA stops in the same sweep: on the decision of sweep s - 3,
+            // every CTA stops in the same sweep: on the decision of sweep s - late,
             // although later ones may be known
             unsigned long long word = 0;
-            if (s >= 3 && lane == 0 && await_decision(s - 3, word) && (word >> 32) &&
-                (int)(word & 0xffffffffull) - 1 == s - 3) {
-                s_stop = s - 3;
+            if (s >= late && lane == 0 && await_decision(s - late, word) && (word >> 32) &&
+                (int)(word & 0xffffffffull) - 1 == s - late) {
+                s_stop = s - late;
                 s_done = (int)(word >> 32);
             }
         }
@@ -530,6 +531,10 @@ int resident_threads() { return RT; }
 cudaError_t launch_resident(const void* fn, int grid, int smem, const DevMat& m, const DevVec& v, const int* cta_row,
                             JacCtl* ctl, int max_sweeps, cudaStream_t s)
 {
+    // the sweeps of a CTA with this much to sum (from 60^3 7-point on, 5.3 us) are longer
+    // than the 3 us in which a decision is taken and read: us a sweep with two / three
+    // sweeps' delay, 64^3 5.91 / 6.01, 70^3 7.04 / 7.08, 27-point 44^3 6.25 / 6.22
+    int late = smem > 128 * 1024 ? 2 : 3;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(RT);
@@ -540,7 +545,7 @@ cudaError_t launch_resident(const void* fn, int grid, int smem, const DevMat& m,
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    void* args[] = {(void*)&m, (void*)&v, (void*)&cta_row, (void*)&ctl, (void*)&max_sweeps};
+    void* args[] = {(void*)&m, (void*)&v, (void*)&cta_row, (void*)&ctl, (void*)&max_sweeps, (void*)&late};
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 

@@ -25,6 +25,28 @@ def _ctas(s):
 
 
 @pytest.mark.parametrize("local", [False, True])
+@pytest.mark.parametrize("name", ["middle", "large", "fe"])
+def test_solves_of_large_systems_stop_at_the_same_sweep(name, local):
+    """Decisions are read three sweeps late in the middle one, two in the others."""
+    A = MATRICES[name][0]()
+    b = np.random.default_rng(6).uniform(-1, 1, A.n)
+    kw = dict(norm=0, stop=J.JAC_STOP_LOCAL, history=2048) if local else dict(history=2048)
+    with J.Solver(A, b, "bandrow", 4, **kw) as a, \
+            J.Solver(A, b, "bandrow", 4, variant=2, ctas_per_sm=2, lanes_per_row=a.stats()["lanes_per_row"], **kw) as p:
+        assert a.stats()["ctas_per_sm"] == 1
+        p.sweep(40)
+        h = p.history()                           # test values of x^0 .. x^39: each ends a solve of its own
+        tols = [1.0001 * h[k] for k in (0, 1, 2, 3, 4, 5, 17)]
+        for maxit, tol in [(1000, t) for t in tols] + [(m, 0.0) for m in (4, 5, 511, 512, 513, 514)]:
+            a.set_x(), p.set_x()
+            ka, kp = a.solve(tol, maxit), p.solve(tol, maxit)
+            assert ka[0] == kp[0] and ka[2] == kp[2] and np.array_equal(a.x(), p.x())
+            ha, hp = a.history(), p.history()
+            assert len(ha) == len(hp) == ka[0] + 1 and np.all(np.abs(ha - hp) <= 2 * A.n * U * hp)
+            assert a.stats()["stop_part"] == p.stats()["stop_part"]
+
+
+@pytest.mark.parametrize("local", [False, True])
 @pytest.mark.parametrize("name", list(MATRICES))
 def test_short_calls_take_the_pipelined_kernel(name, local):
     make, most = MATRICES[name]
