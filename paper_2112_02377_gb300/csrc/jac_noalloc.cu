@@ -122,39 +122,46 @@ __device__ __forceinline__ unsigned shared_addr(const void* p)
 // outside exponents that keep every step normal, and for t = 0, the division itself.
 // 3,374,850 rows, us a sweep: without the tests 92.2, both 93.0, the exact one for
 // every row 96.0, the first alone 96.2 (a warp in 60 divides), IEEE division 105.
-__device__ __forceinline__ double quotient(double t, double d)
+//
+// short_quotient: the value and whether the first test passed; checked_quotient: what
+// holds where it did not.  The kernel stores the first before it knows.
+__device__ __forceinline__ bool short_quotient(double t, double d, double& z)
 {
     const unsigned dh = (unsigned)__double2hiint(d), dl = (unsigned)__double2loint(d);
     const unsigned th = (unsigned)__double2hiint(t);
     const unsigned de = (dh >> 20) & 0x7ffu, te = (th >> 20) & 0x7ffu;
-    if (de - 923u <= 200u && te - 200u <= 1600u) {               // |d| in 2^-100 .. 2^101, |t| in 2^-823 .. 2^778
-        const float f = __uint_as_float((dh & 0x80000000u) | (((dh & 0x7fffffffu) - (896u << 20)) << 3) | (dl >> 29));
-        float rf;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
-        const unsigned rb = __float_as_uint(rf);
-        const double r0 = __hiloint2double((int)((rb & 0x80000000u) | (((rb & 0x7fffffffu) >> 3) + (896u << 20))),
-                                           (int)(rb << 29));
-        const double r = __fma_rn(__fma_rn(-d, r0, 1.0), r0, r0);
-        const double q = __dmul_rn(t, r);
-        const double rem = __fma_rn(-d, q, t);
-        const double z = __fma_rn(rem, r, q);
-        // rem r in ulps of q, in single precision, and the ulps that the rounding took
-        const unsigned mh = (unsigned)__double2hiint(rem), qh = (unsigned)__double2hiint(q);
-        const unsigned zh = (unsigned)__double2hiint(z), zl = (unsigned)__double2loint(z);
-        const unsigned qe = (qh >> 20) & 0x7ffu;
-        const unsigned mb = __funnelshift_l((unsigned)__double2loint(rem), mh & 0x7fffffffu, 3) - ((te - 179u) << 23);
-        // (rem is 0, where z = q is exact and any m will do, or at least 2^-105 |t|)
-        const float m = __uint_as_float(mb | ((mh ^ th) & 0x80000000u));
-        const float c = __fmul_rn(m, __uint_as_float((rb & 0x7fffffffu) + ((te - qe) << 23)));
-        const float off = __fsub_rn(c, (float)(int)(zl - (unsigned)__double2loint(q)));
-        const bool plain = ((zh ^ qh) & 0xfff00000u) == 0 && ((zh & 0xfffffu) | zl) != 0;
-        if (plain && fabsf(off) < 0.4997f) return z;
-        const int back = __double2hiint(__fma_rn(-d, z, t)) & 0x7fffffff;
-        // high word of |d| 2^(e - 53), e the exponent of z (at least 2^-1001)
-        const int half = (int)((dh & 0x7fffffffu) + (zh & 0x7ff00000u) - (1076u << 20));
-        if (back < half && ((zh & 0xfffffu) | zl)) return z;
-    }
-    return t / d;
+    z = 0.0;
+    if (de - 923u > 200u || te - 200u > 1600u) return false;     // |d| in 2^-100 .. 2^101, |t| in 2^-823 .. 2^778
+    const float f = __uint_as_float((dh & 0x80000000u) | (((dh & 0x7fffffffu) - (896u << 20)) << 3) | (dl >> 29));
+    float rf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+    const unsigned rb = __float_as_uint(rf);
+    const double r0 = __hiloint2double((int)((rb & 0x80000000u) | (((rb & 0x7fffffffu) >> 3) + (896u << 20))),
+                                       (int)(rb << 29));
+    const double r = __fma_rn(__fma_rn(-d, r0, 1.0), r0, r0);
+    const double q = __dmul_rn(t, r);
+    const double rem = __fma_rn(-d, q, t);
+    z = __fma_rn(rem, r, q);
+    // rem r in ulps of q, in single precision, and the ulps that the rounding took
+    const unsigned mh = (unsigned)__double2hiint(rem), qh = (unsigned)__double2hiint(q);
+    const unsigned zh = (unsigned)__double2hiint(z), zl = (unsigned)__double2loint(z);
+    const unsigned qe = (qh >> 20) & 0x7ffu;
+    const unsigned mb = __funnelshift_l((unsigned)__double2loint(rem), mh & 0x7fffffffu, 3) - ((te - 179u) << 23);
+    // (rem is 0, where z = q is exact and any m will do, or at least 2^-105 |t|)
+    const float m = __uint_as_float(mb | ((mh ^ th) & 0x80000000u));
+    const float c = __fmul_rn(m, __uint_as_float((rb & 0x7fffffffu) + ((te - qe) << 23)));
+    const float off = __fsub_rn(c, (float)(int)(zl - (unsigned)__double2loint(q)));
+    const bool plain = ((zh ^ qh) & 0xfff00000u) == 0 && ((zh & 0xfffffu) | zl) != 0;
+    return plain && fabsf(off) < 0.4997f;
+}
+
+__device__ __forceinline__ double checked_quotient(double t, double d, double z)
+{
+    const unsigned dh = (unsigned)__double2hiint(d), zh = (unsigned)__double2hiint(z);
+    const int back = __double2hiint(__fma_rn(-d, z, t)) & 0x7fffffff;
+    // high word of |d| 2^(e - 53), e the exponent of z (at least 2^-1001)
+    const int half = (int)((dh & 0x7fffffffu) + (zh & 0x7ff00000u) - (1076u << 20));
+    return back < half && ((zh & 0xfffffu) | (unsigned)__double2loint(z)) ? z : t / d;   // (z = 0: the division)
 }
 
 // One sweep on a CSR matrix that stores its diagonal, one thread per row:
@@ -244,7 +251,12 @@ __global__ void __launch_bounds__(kBlock, 5) k_noalloc_sweep(int n, const int* _
         }
     });
     const double t = bi - s;
-    if (i < n) y[i] = quotient(t, d);
+    if (i < n) {
+        double z;
+        const bool sure = short_quotient(t, d, z);
+        y[i] = z;
+        if (!sure) y[i] = checked_quotient(t, d, z);
+    }
     if constexpr (LAST) {
         double ss = 0.0, mx = 0.0, bb = 0.0;
         if (i < n) {
